@@ -28,6 +28,7 @@
 #include <cudaTypedefs.h>
 
 #include "../../include/sgf.h"
+#include "sgf_block.h"
 #include "sgf_fft16.cuh"
 #include "sgf_host.h"
 #include "sgf_internal.h"
@@ -104,6 +105,8 @@ struct Spectra {
     void *tw = nullptr;    // twiddle area (TwLayout) in the solve precision
     void *twn = nullptr;   // W_N^i, i < N, in the solve precision (register-twiddle kernels)
     int tw_entries = 0;
+    bool blk = false;      // cross-level sets stored for the block convolutions (sgf_block.cuh)
+    void *twb = nullptr;   // twiddle areas of the block transforms (B = 16 .. N/2, blk_tw_offset)
     double plan_ms = 0.0;
 };
 
@@ -116,6 +119,7 @@ void spectra_release(Spectra *s)
         cudaFree(s->dev);
         cudaFree(s->tw);
         cudaFree(s->twn);
+        cudaFree(s->twb);
         cudaSetDevice(cur);
         delete s;
     }
@@ -128,6 +132,17 @@ struct Forest {
     double x0 = 0.0, y0 = 0.0, h0 = 0.0;
     int level[kMaxPatches] = {};
     int org[kMaxPatches][2] = {};  // corner in cells of the patch's level, from (x0, y0)
+};
+
+// Products of one target of a block-convolution stage: per source patch, the
+// kernel blocks (complex offset and strides) and the source's fields.
+struct BlkTarget {
+    struct Term {
+        size_t k_off, sp, sq, x_off;
+    };
+    std::vector<Term> terms;
+    size_t a_off = 0;
+    int m2 = 0, F = 0;
 };
 
 struct SetKey {
@@ -182,6 +197,23 @@ struct sgf_plan {
     int restricted = 0;                         // covered patches (restriction launches per solve)
     std::vector<GenSet> sets;
     size_t fwd_elems = 0, bwd_elems = 0;  // complex elements
+    // cross-level pairs as block convolutions (sgf_block.cuh): the stages (one
+    // per m), their patches, and the products, grouped by kernel spectra.  Their
+    // fields take the place of the forward and column intermediates, which the
+    // patches' own passes are done with by then.
+    bool blk = false;
+    std::vector<BlkStage> stages;
+    std::vector<BlkUnit> bsrc, btgt;
+    std::vector<BlkTarget> btargets;   // products of every target
+    std::vector<MacItem> mitems;
+    std::vector<MacTerm> mterms;
+    std::vector<size_t> mxo, mao;
+    int mac_blocks = 0;
+    size_t blk_x_elems = 0, blk_elems = 0;  // complex elements: source fields; source and target fields
+    const BlkUnit *d_bsrc = nullptr, *d_btgt = nullptr;
+    const MacItem *d_mitems = nullptr;
+    const MacTerm *d_mterms = nullptr;
+    const size_t *d_mxo = nullptr, *d_mao = nullptr;
     // device memory owned by this plan
     void *d_lists = nullptr;
     const FwdSlab *d_slabs = nullptr;
@@ -226,8 +258,8 @@ struct sgf_plan {
     long long inject_wait = 0;
     size_t workspace_bytes = 0;
     size_t algorithmic_bytes = 0;
-    // optional per-kernel timing: 5 events per solve (before restriction, after
-    // restriction, after row_fwd, after col, after row_inv)
+    // optional per-kernel timing: 6 events per solve (before restriction, after
+    // restriction, after row_fwd, after col, after row_inv, after the cross-level pairs)
     bool profile = false;
     std::vector<cudaEvent_t> events;
     size_t events_used = 0;
@@ -249,6 +281,7 @@ struct sgf_batch {
         size_t map_fwd = 0, map_col = 0, map_inv1 = 0, map_inv = 0;  // int2 offsets in the map buffer
         int n_grp = 0, n_sum = 0;
         size_t map_grp = 0, map_sum = 0;  // Case-3 groups (k_col_g), chunked outputs (k_col_sum)
+        bool own = true;  // no finer patch has Case-3 outputs: k_row_inv1 for those too
     };
     std::vector<Group> groups;
     std::vector<int> plan_group;      // group index of every plan
@@ -262,6 +295,13 @@ struct sgf_batch {
     cudaEvent_t uploaded = nullptr;   // after the argument upload of the last solve
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t graph = nullptr;
+    // cross-level pairs (plans with block convolutions): their block arguments, per
+    // pass the first CTA of every such plan, and the products of all of them, plans
+    // that share spectra together
+    int blk_plans = 0, blk_rounds = 0, mac_blocks = 0, mac_items = 0;
+    int blk_blocks[BLK_PASSES + kMaxStages] = {};  // CTAs of the passes, then of the inverse-row rounds
+    void *d_blk = nullptr;
+    size_t off_prefix = 0, off_index = 0, off_items = 0, off_terms = 0, off_xo = 0, off_ao = 0;  // in d_blk
     bool use_graph = true, solved_once = false;
     int launches = 0;                 // kernel launches per solve
 };
@@ -512,6 +552,262 @@ constexpr int kCase3Group = 8;
 // deep nests) is split into chunks that run in parallel.
 constexpr int kChunkInputs = 16;
 
+// ---- cross-level pairs as block convolutions (sgf_block.cuh)
+size_t set_bytes_of(const sgf_plan *p, const GenSet &g);
+
+// Frequencies of a unit's field, B = 2^logB.
+size_t blk_freqs(int logB) { return ((size_t)(1 << logB) + 1) * 2 * ((size_t)1 << logB); }
+
+// Complex elements of one set (one phase of a pair): m^2 blocks of every table.
+size_t blk_set_elems(const sgf_plan *p, const GenSet &g)
+{
+    return (size_t)spec_tables(g.kind) * g.m * g.m * blk_freqs(p->logN - ilog2(g.m));
+}
+
+// Where the block transforms apply: nests (forests) of N >= 256, and blocks of at least 16 cells
+// (the smallest transform) at the plan's depth.  Below 256 the whole-grid
+// passes take fewer launches for transforms that are launch-bound anyway.
+// SGF_BF16X plans of four levels and more stay with the whole-grid passes: the
+// block transforms run in FP32, and from that depth on the split-BF16 rounding
+// they leave out moves the finest level's forces by more than 2e-5 (2-norm;
+// 2.7e-5 at 4 levels, 1.5e-5 at 3, 0.7e-5 at 2).
+bool blk_applies(const sgf_plan *p)
+{
+    return !p->merged && p->fo.depth > 1 && p->N >= 256 && (p->N >> (p->fo.depth - 1)) >= 16 &&
+           !(p->tc && p->fo.depth > 3);
+}
+
+// Twiddle area of the B-point block transforms within Spectra::twb (complex entries).
+int blk_tw_entries(int logB)
+{
+    Fft16Plan pl;
+    pl.init(1 << logB, logB);
+    return tw_layout(pl.twlen, 1 << logB).entries;
+}
+int blk_tw_offset(int logB)
+{
+    int o = 0;
+    for (int l = 4; l < logB; ++l)
+        o += blk_tw_entries(l);
+    return o;
+}
+
+// Target units a warp takes: the accumulators (QG targets, two components, R right-hand
+// sides) have to stay in registers.
+int mac_qg(int qg, int rhs) { return std::min(qg, rhs == 1 ? 4 : rhs == 2 ? 2 : 1); }
+
+// Work items of the products: targets whose terms read the same kernel spectra
+// share them, up to four right-hand sides an item (the accumulators of more do
+// not fit in registers).  QG targets per warp (mac_qg): fewer where the launch would leave SMs without warps
+// (16 warps on each of 152 SMs).  Long items first.
+void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &items, std::vector<MacTerm> &terms,
+               std::vector<size_t> &xo, std::vector<size_t> &ao, int *blocks)
+{
+    std::map<std::vector<size_t>, std::vector<int>> by_k;
+    std::vector<std::vector<size_t>> order;
+    for (int i = 0; i < (int)tg.size(); ++i) {
+        std::vector<size_t> key{(size_t)tg[i].m2, (size_t)tg[i].F};
+        for (const auto &t : tg[i].terms)
+            key.insert(key.end(), {t.k_off, t.sp, t.sq});
+        if (!by_k.count(key))
+            order.push_back(key);
+        by_k[key].push_back(i);
+    }
+    std::stable_sort(order.begin(), order.end(),
+                     [](const std::vector<size_t> &x, const std::vector<size_t> &y) { return x[0] > y[0]; });
+    items.clear();
+    terms.clear();
+    xo.clear();
+    ao.clear();
+    for (const auto &key : order) {
+        const auto &v = by_k[key];
+        for (size_t b = 0; b < v.size(); b += 4) {
+            const int R = (int)std::min<size_t>(4, v.size() - b);
+            const BlkTarget &t0 = tg[v[b]];
+            MacItem it{};
+            it.term_begin = (int)terms.size();
+            it.term_count = (int)t0.terms.size();
+            it.a_begin = (int)ao.size();
+            it.rhs = R;
+            it.m2 = t0.m2;
+            it.F = t0.F;
+            for (size_t k = 0; k < t0.terms.size(); ++k) {
+                terms.push_back(MacTerm{t0.terms[k].k_off, t0.terms[k].sp, t0.terms[k].sq, (int)xo.size(), 0});
+                for (int r = 0; r < R; ++r)
+                    xo.push_back(tg[v[b + r]].terms[k].x_off);
+            }
+            for (int r = 0; r < R; ++r)
+                ao.push_back(tg[v[b + r]].a_off);
+            it.tiles = (it.F / vec + 31) / 32;
+            items.push_back(it);
+        }
+    }
+    int qg = 4;
+    for (; qg > 1; qg >>= 1) {
+        long long warps = 0;
+        for (const auto &it : items)
+            warps += (long long)it.tiles * (it.m2 / mac_qg(qg, it.rhs));
+        if (warps >= 16 * 152)
+            break;
+    }
+    int blk = 0;
+    for (auto &it : items) {
+        it.qg = mac_qg(qg, it.rhs);
+        it.nqg = it.m2 / it.qg;
+        it.blk_begin = blk;
+        const long long warps = (long long)it.tiles * it.nqg;
+        blk += (int)((warps + kBlkThreads / 32 - 1) / (kBlkThreads / 32));
+    }
+    *blocks = blk;
+}
+
+// The stages, sources, targets and products of a plan's cross-level pairs; off:
+// bytes of spectra before theirs.  Sets of one pair (m^2 phases) lie one after
+// the other, pairs of one relative position share them.
+void build_blocks(sgf_plan *p, size_t off)
+{
+    const Forest &fo = p->fo;
+    const size_t Cb = 2 * p->esize;
+    std::map<SetKey, int> group;  // first set of a pair's m^2 phases
+    auto get_group = [&](int cas, int m, int ax, int ay, int fine) {
+        SetKey key{cas, m, 0, 0, ax, ay, p->pot ? fine : 0};
+        auto it = group.find(key);
+        if (it != group.end())
+            return it->second;
+        const int first = (int)p->sets.size();
+        for (int py = 0; py < m; ++py)
+            for (int px = 0; px < m; ++px) {
+                GenSet g{};
+                g.kind = p->pot ? SPEC_FULL_PHI : SPEC_FULL;
+                g.cas = cas;
+                g.m = m;
+                g.px = px;
+                g.py = py;
+                g.ax = ax;
+                g.ay = ay;
+                g.h = p->pot ? std::ldexp(fo.h0, -fine) : 0.0;
+                g.spec_off = off / Cb;
+                off += set_bytes_of(p, g);
+                p->sets.push_back(g);
+            }
+        group[key] = first;
+        return first;
+    };
+    const int nc = p->pot ? 1 : 2;
+    size_t x = 0, acc = 0;
+    for (int d = 1; d < fo.depth; ++d) {
+        BlkStage sg{};
+        sg.m = 1 << d;
+        sg.logB = p->logN - d;
+        const size_t F = blk_freqs(sg.logB), m2 = (size_t)sg.m * sg.m;
+        sg.src_begin = (int)p->bsrc.size();
+        sg.tgt_begin = (int)p->btgt.size();
+        sg.x_off = x;
+        sg.a_off = acc;
+        sg.tw_off = blk_tw_offset(sg.logB);
+        sg.tw_entries = blk_tw_entries(sg.logB);
+        size_t x_of[2][kMaxPatches];
+        for (int kind = 0; kind < 2; ++kind)  // phases of the finer patches, blocks of the coarser
+            for (int s = 0; s < fo.K; ++s)
+                if (kind == 0 ? fo.level[s] >= d : fo.level[s] + d < fo.depth) {
+                    x_of[kind][s] = x;
+                    x += 3 * m2 * F;
+                    p->bsrc.push_back(BlkUnit{s, kind});
+                    sg.src_count++;
+                }
+        for (int kind = 0; kind < 2; ++kind)
+            for (int t = 0; t < fo.K; ++t)
+                if (kind == 0 ? fo.level[t] + d < fo.depth : fo.level[t] >= d) {
+                    BlkTarget bt;
+                    bt.a_off = acc;
+                    bt.m2 = (int)m2;
+                    bt.F = (int)F;
+                    for (int s = 0; s < fo.K; ++s) {
+                        if (fo.level[s] != fo.level[t] + (kind == 0 ? d : -d))
+                            continue;
+                        const int fi = kind == 0 ? s : t, co = kind == 0 ? t : s;  // finer, coarser
+                        const int g = get_group(kind == 0 ? kBlkCase2 : kBlkCase3, sg.m, fo.org[fi][0] - fo.org[co][0] * sg.m,
+                                                fo.org[fi][1] - fo.org[co][1] * sg.m, fo.level[fi]);
+                        const GenSet &g0 = p->sets[g];
+                        const size_t per_set = set_bytes_of(p, g0) / Cb, per_blk = (size_t)spec_tables(g0.kind) * F;
+                        // set = phase (source of Case 2, target of Case 3), block = the other side
+                        bt.terms.push_back({g0.spec_off, kind == 0 ? per_set : per_blk, kind == 0 ? per_blk : per_set,
+                                            x_of[kind][s]});
+                    }
+                    acc += nc * m2 * F;
+                    p->btgt.push_back(BlkUnit{t, kind});
+                    sg.tgt_count[kind]++;
+                    p->btargets.push_back(bt);
+                }
+        p->stages.push_back(sg);
+    }
+    p->blk_x_elems = x;
+    p->blk_elems = x + acc;
+    build_mac(p->btargets, p->esize == 8 ? 1 : 2, p->mitems, p->mterms, p->mxo, p->mao, &p->mac_blocks);
+}
+
+// Block arguments of a solve whose source and target fields start at `work`.
+template <typename T>
+void fill_blk(const sgf_plan *p, void *work, BlkArgs<T> &k)
+{
+    using C = typename BlkArgs<T>::C;
+    k.stages = (int)p->stages.size();
+    for (int pass = 0; pass < BLK_PASSES; ++pass) {
+        int b = 0;
+        for (int i = 0; i < k.stages; ++i) {
+            k.blocks[pass][i] = b;
+            b += blk_blocks(pass, p->stages[i], p->pot ? 1 : 2);
+        }
+        k.blocks[pass][k.stages] = b;
+    }
+    for (int i = 0; i < k.stages; ++i)
+        k.st[i] = p->stages[i];
+    // inverse rows, round r: every patch's pair with the r-th of the other levels
+    k.rounds = p->fo.depth - 1;
+    for (int r = 0; r < k.rounds; ++r) {
+        int n = 0, b = 0;
+        for (int t = 0; t < p->fo.K; ++t) {
+            const int lt = p->fo.level[t], ls = r < lt ? r : r + 1, kind = ls > lt ? 0 : 1;
+            const int stage = std::abs(ls - lt) - 1;
+            const BlkStage &sg = p->stages[stage];
+            int ti = 0;
+            while (p->btgt[sg.tgt_begin + ti].patch != t || p->btgt[sg.tgt_begin + ti].kind != kind)
+                ++ti;
+            k.seg[r][n++] = BlkSeg{stage, ti, b};
+            b += blk_blocks(BLK_IROWS, sg, p->pot ? 1 : 2);
+        }
+        k.segs[r] = n;
+        k.seg[r][n] = BlkSeg{0, 0, b};
+    }
+    k.src = p->d_bsrc;
+    k.tgt = p->d_btgt;
+    k.tw = static_cast<const C *>(p->spec->twb);
+    k.x = static_cast<C *>(work);
+    k.acc = k.x + p->blk_x_elems;
+}
+
+// The cross-level pairs of a solve, added to the forces (or the potential) that the
+// patches' own passes have stored.
+template <typename T>
+cudaError_t launch_blocks(const sgf_plan *p, const SolveArgs<T> &a, void *work, cudaStream_t st)
+{
+    BlkArgs<T> k{};
+    fill_blk<T>(p, work, k);
+    auto pass = [&](int ps) { return launch_blk_pass<T>(ps, 0, k.blocks[ps][k.stages], a, k, st); };
+    cudaError_t e;
+    if ((e = pass(BLK_ROWS)) != cudaSuccess || (e = pass(BLK_COLS)) != cudaSuccess)
+        return e;
+    if ((e = launch_blk_mac<T>(p->mac_blocks, p->d_mitems, (int)p->mitems.size(), p->d_mterms, p->d_mxo, p->d_mao,
+                               p->spec->dev, k.x, k.acc, a.ncomp, st)) != cudaSuccess)
+        return e;
+    if ((e = pass(BLK_ICOLS)) != cudaSuccess)
+        return e;
+    for (int r = 0; r < k.rounds; ++r)
+        if ((e = launch_blk_pass<T>(BLK_IROWS, r, k.seg[r][k.segs[r]].blk, a, k, st)) != cudaSuccess)
+            return e;
+    return cudaSuccess;
+}
+
 // Build all host-side lists of a plan (no CUDA calls).  Every ordered pair of
 // patches (source s, target t) contributes:
 //   same patch              Case 1, the shared quarter-stored set
@@ -519,6 +815,9 @@ constexpr int kChunkInputs = 16;
 //                           run as Case 2 with m = 1 (a full complex set)
 //   s finer (Case 2)        m^2 source phases into t's main output
 //   s coarser (Case 3)      m^2 target-phase outputs of N/m rows each
+//
+// p->blk: the pairs of different levels run as block convolutions instead
+// (build_blocks), the patches' own outputs as above.
 void build_lists(sgf_plan *p)
 {
     if (p->merged) {
@@ -571,7 +870,7 @@ void build_lists(sgf_plan *p)
         slab_full[s] = add_slab(s, 1, 0, 0);
     for (int s = 0; s < L; ++s)
         for (int t = 0; t < L; ++t) {
-            if (fo.level[s] <= fo.level[t])
+            if (p->blk || fo.level[s] <= fo.level[t])
                 continue;
             const int m = 1 << (fo.level[s] - fo.level[t]);
             for (int py = 0; py < m; ++py)
@@ -613,7 +912,7 @@ void build_lists(sgf_plan *p)
         }
         for (int s = 0; s < L; ++s) {  // Case 2: finer sources, A = corner_s - corner_t in s cells
             const int ls = fo.level[s];
-            if (ls <= lt)
+            if (p->blk || ls <= lt)
                 continue;
             const int m = 1 << (ls - lt);
             const int ax = fo.org[s][0] - fo.org[t][0] * m, ay = fo.org[s][1] - fo.org[t][1] * m;
@@ -623,7 +922,7 @@ void build_lists(sgf_plan *p)
         }
         for (int s = 0; s < L; ++s) {  // Case 3: coarser sources, one output per target phase
             const int ls = fo.level[s];
-            if (ls >= lt)
+            if (p->blk || ls >= lt)
                 continue;
             const int m = 1 << (lt - ls);
             const int ax = fo.org[t][0] - fo.org[s][0] * m, ay = fo.org[t][1] - fo.org[s][1] * m;
@@ -641,7 +940,7 @@ void build_lists(sgf_plan *p)
         p->contrib_begin[t] = (int)p->contribs.size();
         p->contribs.push_back(RowContrib{1, 0, main_out[t], 0});
         for (int s = 0; s < L; ++s) {
-            if (fo.level[s] >= fo.level[t])
+            if (p->blk || fo.level[s] >= fo.level[t])
                 continue;
             const int m = 1 << (fo.level[t] - fo.level[s]);
             for (int px = 0; px < m; ++px)
@@ -670,7 +969,7 @@ void build_lists(sgf_plan *p)
             p->work_all.push_back(ColWork{o, p->outs[o].in_begin, p->outs[o].in_count, -1});
     for (int t = 0; t < L; ++t) {
         for (int s = 0; s < L; ++s) {  // sub-groups of at most kCase3Group outputs keep the columns parallel
-            if (fo.level[s] >= fo.level[t])
+            if (p->blk || fo.level[s] >= fo.level[t])
                 continue;
             const int m = 1 << (fo.level[t] - fo.level[s]);
             for (int q = 0; q < m * m; q += kCase3Group)
@@ -682,13 +981,13 @@ void build_lists(sgf_plan *p)
         for (int r = 0; r < p->slabs[k].rows / 2; ++r)
             p->items.push_back(FwdItem{k, r});
     // spectra offsets: 256-byte aligned sets in one buffer
-    std::vector<size_t> set_off(p->sets.size());
     size_t off = 0;
     for (size_t k = 0; k < p->sets.size(); ++k) {
-        set_off[k] = off;
+        p->sets[k].spec_off = spec_quarter(p->sets[k].kind) ? off / T : off / Cb;
         off += (set_bytes[k] + 255) & ~(size_t)255;
-        p->sets[k].spec_off = spec_quarter(p->sets[k].kind) ? set_off[k] / T : set_off[k] / Cb;
     }
+    if (p->blk)
+        build_blocks(p, off);
     p->in_set.clear();
     for (auto &ci : p->ins) {
         p->in_set.push_back((int)ci.spec_off);
@@ -712,31 +1011,61 @@ void build_lists(sgf_plan *p)
                 cov += (size_t)(p->cover[k].x1 - p->cover[k].x0) * (p->cover[k].y1 - p->cover[k].y0);
             ab += 2 * (size_t)N * N * T + 4 * cov * T;
         }
+    // block convolutions: every source and target field written and read twice (rows, columns), the
+    // kernel spectra of every pair read once, the forces read and written where a pair adds to them
+    for (const auto &sg : p->stages) {
+        const size_t fld = (size_t)sg.m * sg.m * blk_freqs(sg.logB) * Cb;
+        ab += 3 * fld * 3 * sg.src_count + ncomp * fld * 3 * (sg.tgt_count[0] + sg.tgt_count[1]) +
+              2 * ncomp * (size_t)N * N * T * (sg.tgt_count[0] + sg.tgt_count[1]);
+    }
+    for (const auto &bt : p->btargets)
+        ab += bt.terms.size() * (size_t)bt.m2 * bt.m2 * 3 * ncomp * bt.F * Cb;
     p->algorithmic_bytes = ab;
-    (void)off;
+}
+
+// Stored bytes of one spectra set (256-byte aligned).
+size_t set_bytes_of(const sgf_plan *p, const GenSet &g)
+{
+    const size_t nt = (size_t)spec_tables(g.kind);
+    const size_t b = gen_blk(g) ? blk_set_elems(p, g) * 2 * p->esize
+                     : g.kind == SPEC_MERGED || g.kind == SPEC_MERGED_PHI || spec_quarter(g.kind)
+                         ? nt * (p->N + 1) * quarter_stride(p->N) * p->esize
+                         : nt * (p->N + 1) * 2 * p->N * 2 * p->esize;
+    return (b + 255) & ~(size_t)255;
 }
 
 size_t spectra_total(const sgf_plan *p)
 {
     size_t off = 0;
-    for (const auto &g : p->sets) {
-        const size_t nt = (size_t)spec_tables(g.kind);
-        const size_t b = g.kind == SPEC_MERGED || g.kind == SPEC_MERGED_PHI || spec_quarter(g.kind)
-                             ? nt * (p->N + 1) * quarter_stride(p->N) * p->esize
-                             : nt * (p->N + 1) * 2 * p->N * 2 * p->esize;
-        off += (b + 255) & ~(size_t)255;
-    }
+    for (const auto &g : p->sets)
+        off += set_bytes_of(p, g);
     return off;
 }
 
-// Stored bytes of one spectra set (256-byte aligned), as spectra_total counts them.
-size_t set_bytes_of(const sgf_plan *p, const GenSet &g)
+// Empties what build_lists fills.
+void reset_lists(sgf_plan *p)
 {
-    const size_t nt = (size_t)spec_tables(g.kind);
-    const size_t b = g.kind == SPEC_MERGED || g.kind == SPEC_MERGED_PHI || spec_quarter(g.kind)
-                         ? nt * (p->N + 1) * quarter_stride(p->N) * p->esize
-                         : nt * (p->N + 1) * 2 * p->N * 2 * p->esize;
-    return (b + 255) & ~(size_t)255;
+    p->slabs.clear();
+    p->items.clear();
+    p->outs.clear();
+    p->ins.clear();
+    p->contribs.clear();
+    p->work_all.clear();
+    p->work_main.clear();
+    p->groups.clear();
+    p->sums.clear();
+    p->sets.clear();
+    p->in_set.clear();
+    p->stages.clear();
+    p->bsrc.clear();
+    p->btgt.clear();
+    p->btargets.clear();
+    p->mitems.clear();
+    p->mterms.clear();
+    p->mxo.clear();
+    p->mao.clear();
+    p->partial_elems = p->fwd_elems = p->bwd_elems = p->blk_x_elems = p->blk_elems = 0;
+    p->mac_blocks = 0;
 }
 
 // A plan whose kernel spectra exceed its budget.  Residency: the sets of the
@@ -753,10 +1082,18 @@ size_t set_bytes_of(const sgf_plan *p, const GenSet &g)
 // The Case-3 groups of k_col_g are not used (each Case-3 output is its own work item).
 sgf_status plan_stream_layout(sgf_plan *p)
 {
-    const size_t total = spectra_total(p);
+    size_t total = spectra_total(p);
     p->streamed = false;
     if (p->spectra_budget == 0 || total <= p->spectra_budget)
         return SGF_OK;
+    if (p->blk) {  // streamed sets are those of the whole-grid passes
+        reset_lists(p);
+        p->blk = false;
+        build_lists(p);
+        total = spectra_total(p);
+        if (total <= p->spectra_budget)
+            return SGF_OK;
+    }
     if (p->merged || p->pot)
         return fail(SGF_EUNSUPPORTED,
                     "a spectra budget below the plan's %zu bytes of spectra needs a force plan without "
@@ -881,8 +1218,7 @@ void plan_free_owned(sgf_plan *p)
     cudaGetDevice(&cur);
     cudaSetDevice(p->device);
     cudaFree(p->d_lists);
-    cudaFree(p->d_fwd);
-    cudaFree(p->d_bwd);
+    cudaFree(p->d_fwd);  // d_bwd lies in the same allocation
     cudaFree(p->d_restricted);
     cudaFree(p->d_stage);
     cudaFree(p->d_pipe);
@@ -929,6 +1265,17 @@ size_t io_stage_bytes(const sgf_plan *p)
     return p->n_log == p->N ? 0 : (size_t)(p->pot ? 2 : 3) * p->L * p->N * p->N * p->esize;
 }
 
+size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// Bytes of a solve's intermediates: the forward slabs and behind them the column
+// outputs, and, once the patches' own passes are done with those, the fields of the
+// block convolutions.
+size_t inter_bytes(const sgf_plan *p)
+{
+    const size_t Cb = 2 * p->esize;
+    return std::max(align256(p->fwd_elems * Cb) + p->bwd_elems * Cb, p->blk_elems * Cb);
+}
+
 // Device bytes plan_alloc_owned allocates for p (lists, intermediates, restricted densities).
 size_t workspace_of(const sgf_plan *p)
 {
@@ -943,7 +1290,13 @@ size_t workspace_of(const sgf_plan *p)
     align_push(blob, p->groups);
     align_push(blob, p->sums);
     align_push(blob, p->work_stream);
-    return blob.size() + p->partial_elems * 2 * p->esize + (p->fwd_elems + p->bwd_elems) * 2 * p->esize +
+    align_push(blob, p->bsrc);
+    align_push(blob, p->btgt);
+    align_push(blob, p->mitems);
+    align_push(blob, p->mterms);
+    align_push(blob, p->mxo);
+    align_push(blob, p->mao);
+    return blob.size() + p->partial_elems * 2 * p->esize + inter_bytes(p) +
            (size_t)p->restricted * p->N * p->N * p->esize + (p->streamed ? gen_bytes_of(p->N) : 0) +
            io_stage_bytes(p);
 }
@@ -1000,6 +1353,12 @@ sgf_status plan_alloc_owned(sgf_plan *p)
     const size_t o_grp = align_push(blob, p->groups);
     const size_t o_sum = align_push(blob, p->sums);
     const size_t o_str = align_push(blob, p->work_stream);
+    const size_t o_bsrc = align_push(blob, p->bsrc);
+    const size_t o_btgt = align_push(blob, p->btgt);
+    const size_t o_mi = align_push(blob, p->mitems);
+    const size_t o_mt = align_push(blob, p->mterms);
+    const size_t o_mx = align_push(blob, p->mxo);
+    const size_t o_ma = align_push(blob, p->mao);
     cudaError_t e;
     if ((e = cudaMalloc(&p->d_lists, blob.size())) != cudaSuccess)
         return cuda_fail(e, "cudaMalloc(work lists)");
@@ -1016,6 +1375,12 @@ sgf_status plan_alloc_owned(sgf_plan *p)
     p->d_groups = reinterpret_cast<const ColGroup *>(base + o_grp);
     p->d_sums = reinterpret_cast<const ColSum *>(base + o_sum);
     p->d_work_stream = reinterpret_cast<const ColWork *>(base + o_str);
+    p->d_bsrc = reinterpret_cast<const BlkUnit *>(base + o_bsrc);
+    p->d_btgt = reinterpret_cast<const BlkUnit *>(base + o_btgt);
+    p->d_mitems = reinterpret_cast<const MacItem *>(base + o_mi);
+    p->d_mterms = reinterpret_cast<const MacTerm *>(base + o_mt);
+    p->d_mxo = reinterpret_cast<const size_t *>(base + o_mx);
+    p->d_mao = reinterpret_cast<const size_t *>(base + o_ma);
     if (p->streamed) {  // the window of the streamed sets and the generator's workspace, for every solve
         if ((e = cudaMalloc(&p->d_window, p->window_bytes)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc(spectra window)");
@@ -1035,10 +1400,9 @@ sgf_status plan_alloc_owned(sgf_plan *p)
     const size_t Cb = 2 * p->esize;
     if (p->partial_elems && (e = cudaMalloc(&p->d_partial, p->partial_elems * Cb)) != cudaSuccess)
         return cuda_fail(e, "cudaMalloc(chunk accumulators)");
-    if ((e = cudaMalloc(&p->d_fwd, p->fwd_elems * Cb)) != cudaSuccess)
-        return cuda_fail(e, "cudaMalloc(forward intermediates)");
-    if ((e = cudaMalloc(&p->d_bwd, p->bwd_elems * Cb)) != cudaSuccess)
-        return cuda_fail(e, "cudaMalloc(backward intermediates)");
+    if ((e = cudaMalloc(&p->d_fwd, inter_bytes(p))) != cudaSuccess)
+        return cuda_fail(e, "cudaMalloc(intermediates)");
+    p->d_bwd = static_cast<unsigned char *>(p->d_fwd) + align256(p->fwd_elems * Cb);
     if (p->restricted > 0) {
         if ((e = cudaMalloc(&p->d_restricted, (size_t)p->restricted * p->N * p->N * p->esize)) != cudaSuccess)
             return cuda_fail(e, "cudaMalloc(restricted densities)");
@@ -1076,43 +1440,43 @@ void twiddles(int P, std::vector<double> &re, std::vector<double> &im)
 }
 
 // Transient device memory of the table generator (FP64 tables, half spectra, twiddles).
-size_t gen_workspace_bytes(int N)
+// (block convolutions at depth > 1: half spectra of m^2 blocks of B + 1 bins, and the
+// twiddles of every B)
+size_t gen_half_elems(const sgf_plan *p)
 {
-    const size_t P = 2 * (size_t)N;
-    return 6 * P * P * sizeof(double) + 6 * (size_t)(N + 1) * P * sizeof(double2) + P * sizeof(double2);
+    const size_t rows = p->blk ? (size_t)p->N + ((size_t)1 << (p->fo.depth - 1)) : (size_t)p->N + 1;
+    return 6 * rows * 2 * p->N;
+}
+size_t gen_tw_elems(const sgf_plan *p) { return (p->blk ? 4 : 2) * (size_t)p->N; }
+size_t gen_workspace_bytes(const sgf_plan *p)
+{
+    const size_t P = 2 * (size_t)p->N;
+    return 6 * P * P * sizeof(double) + gen_half_elems(p) * sizeof(double2) + gen_tw_elems(p) * sizeof(double2);
 }
 
-template <typename T>
-sgf_status build_spectra(sgf_plan *p)
+// Twiddle area (tw_layout) of the transforms of N = 2^logN points, from W_Q^k, k < Q = re.size()
+// (a multiple of 2N): stage tables W_{R Ns}^{r k}, then W_P^j, then W_32^u (P = 2N).
+template <typename C>
+std::vector<C> solve_twiddles(int logN, const std::vector<double> &re, const std::vector<double> &im)
 {
-    using C = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
-    const int N = p->N, P = 2 * N;
-    auto t0 = std::chrono::steady_clock::now();
-    Spectra *sp = new Spectra();
-    sp->device = p->device;
-    p->spec = sp;
-    cudaError_t e;
-    std::vector<double> re, im;
-    twiddles(P, re, im);
-    std::vector<double2> tw64(P);
-    for (int k = 0; k < P; ++k)
-        tw64[k] = make_double2(re[k], im[k]);
-    // solve twiddle area: stage tables W_{R Ns}^{r k} = W_P^{2N r k / (R Ns)}, then W_P^j, then W_32^u
+    using T = typename Real<C>::T;
+    const int N = 1 << logN;
+    const long P = 2L * N, up = (long)re.size() / P;
     Fft16Plan pl;
-    pl.init(N, p->logN);
+    pl.init(N, logN);
     const TwLayout tl = tw_layout(pl.twlen, N);
-    std::vector<C> twT(tl.entries);
-    for (auto &c : twT)
+    std::vector<C> tw(tl.entries);
+    for (auto &c : tw)
         c.x = c.y = (T)0;
     auto put = [&](int at, long idx) {
         idx %= P;
-        twT[at].x = (T)re[idx];
-        twT[at].y = (T)im[idx];
+        tw[at].x = (T)re[idx * up];
+        tw[at].y = (T)im[idx * up];
     };
     // W_{R Ns}^{e} = W_P^{e 2N / (R Ns)}; layout per Fft16Plan (direct or factored over k = 16 kh + kl)
     for (int st = 1, Ns = pl.radix(0); st < pl.nst; Ns *= pl.radix(st), ++st) {
         const int R = pl.radix(st);
-        const long scale = (long)2 * N / ((long)R * Ns);
+        const long scale = P / ((long)R * Ns);
         const int t0 = pl.twoff[st];
         for (int r = 1; r < R; ++r) {
             if (Ns < 256) {
@@ -1130,11 +1494,46 @@ sgf_status build_spectra(sgf_plan *p)
         put(tl.base + jj, jj);
     for (int u = 0; u < 16; ++u)
         put(tl.w32 + u, (long)u * (P / 32));
-    sp->tw_entries = tl.entries;
-    if ((e = cudaMalloc(&sp->tw, tl.entries * sizeof(C))) != cudaSuccess)
+    return tw;
+}
+
+template <typename T>
+sgf_status build_spectra(sgf_plan *p)
+{
+    using C = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
+    const int N = p->N, P = 2 * N;
+    auto t0 = std::chrono::steady_clock::now();
+    Spectra *sp = new Spectra();
+    sp->blk = p->blk;
+    sp->device = p->device;
+    p->spec = sp;
+    cudaError_t e;
+    std::vector<double> re, im;
+    twiddles(P, re, im);
+    std::vector<double2> tw64(gen_tw_elems(p), make_double2(0.0, 0.0));
+    for (int k = 0; k < P; ++k)
+        tw64[k] = make_double2(re[k], im[k]);
+    for (size_t m = 2, o = P; p->blk && m <= ((size_t)1 << (p->fo.depth - 1)); o += P / m, m <<= 1)
+        for (size_t k = 0; k < P / m; ++k)  // W_{P/m}^k
+            tw64[o + k] = tw64[k * m];
+    // solve twiddle area: stage tables W_{R Ns}^{r k} = W_P^{2N r k / (R Ns)}, then W_P^j, then W_32^u
+    const std::vector<C> twT = solve_twiddles<C>(p->logN, re, im);
+    sp->tw_entries = (int)twT.size();
+    if ((e = cudaMalloc(&sp->tw, twT.size() * sizeof(C))) != cudaSuccess)
         return cuda_fail(e, "cudaMalloc(twiddles)");
-    if ((e = upload_landed(sp->tw, twT.data(), tl.entries * sizeof(C))) != cudaSuccess)
+    if ((e = upload_landed(sp->tw, twT.data(), twT.size() * sizeof(C))) != cudaSuccess)
         return cuda_fail(e, "cudaMemcpy(twiddles)");
+    if (p->blk) {  // one area per block size, as blk_tw_offset lays them out
+        std::vector<C> twb;
+        for (int l = 4; l < p->logN; ++l) {
+            const std::vector<C> t = solve_twiddles<C>(l, re, im);
+            twb.insert(twb.end(), t.begin(), t.end());
+        }
+        if ((e = cudaMalloc(&sp->twb, twb.size() * sizeof(C))) != cudaSuccess)
+            return cuda_fail(e, "cudaMalloc(block twiddles)");
+        if ((e = upload_landed(sp->twb, twb.data(), twb.size() * sizeof(C))) != cudaSuccess)
+            return cuda_fail(e, "cudaMemcpy(block twiddles)");
+    }
     {  // the full table W_N^i = W_P^{2i} of the register-twiddle kernels
         std::vector<C> twn(N);
         for (int i = 0; i < N; ++i) {
@@ -1153,10 +1552,10 @@ sgf_status build_spectra(sgf_plan *p)
     double *d_tables = nullptr;
     double2 *d_half = nullptr;
     sgf_status st = SGF_OK;
-    if ((e = cudaMalloc(&d_tw64, P * sizeof(double2))) != cudaSuccess ||
-        (e = upload_landed(d_tw64, tw64.data(), P * sizeof(double2))) != cudaSuccess ||
+    if ((e = cudaMalloc(&d_tw64, tw64.size() * sizeof(double2))) != cudaSuccess ||
+        (e = upload_landed(d_tw64, tw64.data(), tw64.size() * sizeof(double2))) != cudaSuccess ||
         (e = cudaMalloc(&d_tables, 6 * (size_t)P * P * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&d_half, 6 * (size_t)(N + 1) * P * sizeof(double2))) != cudaSuccess) {
+        (e = cudaMalloc(&d_half, gen_half_elems(p) * sizeof(double2))) != cudaSuccess) {
         st = cuda_fail(e, "cudaMalloc(table generation workspace)");
     }
     if (st == SGF_OK && (e = gen_kernels_init()) != cudaSuccess)
@@ -1208,7 +1607,7 @@ sgf_status mark(sgf_plan *p, cudaStream_t st)
 // 5: k_row_inv2x, whose map of two row pairs a box (tmap2) replaces a.tmap_inv.
 template <typename T>
 cudaError_t launch_row_inv(int logN, int L, int R, SolveArgs<T> a, cudaStream_t st, bool tc, int row_inv0,
-                           int inv_radix = 0, const unsigned char *tmap2 = nullptr)
+                           int inv_radix = 0, const unsigned char *tmap2 = nullptr, bool own = false)
 {
     a.level_base = 0;
     if (row_inv0 == 1)
@@ -1227,6 +1626,8 @@ cudaError_t launch_row_inv(int logN, int L, int R, SolveArgs<T> a, cudaStream_t 
     if (e != cudaSuccess || L == R)
         return e;
     a.level_base = R;
+    if (own)  // the finer patches have their own main output alone as well (block convolutions)
+        return launch_pass_n<T>(row_inv0 == 2 ? PASS_ROW_INV2 : PASS_ROW_INV1, logN, a, L - R, st, nullptr, tc);
     return launch_pass_n<T>(PASS_ROW_INV, logN, a, L - R, st, nullptr, tc);
 }
 
@@ -1435,9 +1836,13 @@ sgf_status solve_core(sgf_plan *p, const void *const *sigma, void *const *fx, vo
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
     if ((e = launch_row_inv<T>(p->logN, L, p->fo.R, a, st, p->tc, p->sched.row_inv0, p->sched.inv_radix,
-                               p->tmap_inv2)) !=
+                               p->tmap_inv2, p->blk)) !=
         cudaSuccess)
         return cuda_fail(e, "row_inv launch");
+    if ((ms = mark(p, st)) != SGF_OK)
+        return ms;
+    if (p->blk && (e = launch_blocks<T>(p, a, p->d_fwd, st)) != cudaSuccess)
+        return cuda_fail(e, "block convolution launch");
     return mark(p, st);
 }
 
@@ -1544,14 +1949,12 @@ sgf_status solve_dispatch(sgf_plan *p, const void *const *sigma, void *const *fx
 // creation keeps that reservation out of the call that promises not to allocate.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SGF_NOALLOC_SCRATCH_BYTES];
 
-size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
-
-// Bytes of scratch a plan's solve needs: restricted densities, forward and backward intermediates.
+// Bytes of scratch a plan's solve needs: restricted densities, intermediates, chunk accumulators.
 size_t noalloc_bytes(const sgf_plan *p)
 {
     const size_t Cb = 2 * p->esize;
-    return align256((size_t)p->restricted * p->N * p->N * p->esize) + align256(p->fwd_elems * Cb) +
-           align256(p->bwd_elems * Cb) + align256(p->partial_elems * Cb);
+    return align256((size_t)p->restricted * p->N * p->N * p->esize) + align256(inter_bytes(p)) +
+           align256(p->partial_elems * Cb);
 }
 
 // The scratch array's device address in the current context (the plan's
@@ -1577,7 +1980,7 @@ sgf_status solve_noalloc_impl(sgf_plan *p, const void *const *sigma, void *const
     T *restricted = reinterpret_cast<T *>(scratch);
     unsigned char *fwd = scratch + align256((size_t)p->restricted * N * N * p->esize);
     unsigned char *bwd = fwd + align256(p->fwd_elems * Cb);
-    unsigned char *partial = bwd + align256(p->bwd_elems * Cb);
+    unsigned char *partial = fwd + align256(inter_bytes(p));
     SolveArgs<T> a{};
     fill_geometry(p, a);
     cudaError_t er = fill_sources<T>(p, sigma, restricted, a, true, st);
@@ -1614,8 +2017,10 @@ sgf_status solve_noalloc_impl(sgf_plan *p, const void *const *sigma, void *const
         return cuda_fail(e, "col launch");
     // the plan's tensor map points at its own intermediates, not at the scratch array
     const int inv0 = p->sched.row_inv0 >= 3 ? 0 : p->sched.row_inv0;
-    if ((e = launch_row_inv<T>(p->logN, L, p->fo.R, a, st, p->tc, inv0)) != cudaSuccess)
+    if ((e = launch_row_inv<T>(p->logN, L, p->fo.R, a, st, p->tc, inv0, 0, nullptr, p->blk)) != cudaSuccess)
         return cuda_fail(e, "row_inv launch");
+    if (p->blk && (e = launch_blocks<T>(p, a, fwd, st)) != cudaSuccess)
+        return cuda_fail(e, "block convolution launch");
     if ((e = cudaEventRecord(p->done, st)) != cudaSuccess)
         return cuda_fail(e, "cudaEventRecord(solve completion)");
     return SGF_OK;
@@ -1711,10 +2116,102 @@ sgf_status batch_launches(sgf_batch *bt, cudaStream_t st)
             if ((e = launch_pass_n<T>(g.sched.row_inv0 == 2 ? PASS_ROW_INV2 : PASS_ROW_INV1, g.logN, dummy, g.n_inv1,
                                       gs, &vi1, g.tc)) != cudaSuccess)
                 return cuda_fail(e, "batched row_inv1 launch");
-            if (g.n_inv > 0 && (e = launch_pass_n<T>(PASS_ROW_INV, g.logN, dummy, g.n_inv, gs, &vi, g.tc)) != cudaSuccess)
+            const int fine = !g.own                  ? PASS_ROW_INV
+                             : g.sched.row_inv0 == 2 ? PASS_ROW_INV2
+                                                     : PASS_ROW_INV1;
+            if (g.n_inv > 0 && (e = launch_pass_n<T>(fine, g.logN, dummy, g.n_inv, gs, &vi, g.tc)) != cudaSuccess)
                 return cuda_fail(e, "batched row_inv launch");
         }
     }
+    if (bt->blk_plans > 0) {  // the cross-level pairs of every plan, as launch_blocks
+        using C = typename BlkArgs<T>::C;
+        const unsigned char *base = static_cast<const unsigned char *>(bt->d_blk);
+        const BlkArgs<T> *dk = reinterpret_cast<const BlkArgs<T> *>(base);
+        const int *prefix = reinterpret_cast<const int *>(base + bt->off_prefix);
+        const int *index = reinterpret_cast<const int *>(base + bt->off_index);
+        auto pass = [&](int ps, int round = 0) {
+            return launch_blk_pass_batch<T>(ps, round, bt->blk_blocks[ps + round], bt->blk_plans,
+                                            prefix + (size_t)(ps + round) * (bt->blk_plans + 1), index, args, dk, st);
+        };
+        if ((e = pass(BLK_ROWS)) != cudaSuccess || (e = pass(BLK_COLS)) != cudaSuccess ||
+            (e = launch_blk_mac<T>(bt->mac_blocks, reinterpret_cast<const MacItem *>(base + bt->off_items),
+                                   bt->mac_items, reinterpret_cast<const MacTerm *>(base + bt->off_terms),
+                                   reinterpret_cast<const size_t *>(base + bt->off_xo),
+                                   reinterpret_cast<const size_t *>(base + bt->off_ao), static_cast<const C *>(nullptr),
+                                   static_cast<const C *>(nullptr), static_cast<C *>(nullptr), 2, st)) != cudaSuccess ||
+            (e = pass(BLK_ICOLS)) != cudaSuccess)
+            return cuda_fail(e, "batched block convolution launch");
+        for (int r = 0; r < bt->blk_rounds; ++r)
+            if ((e = pass(BLK_IROWS, r)) != cudaSuccess)
+                return cuda_fail(e, "batched block convolution launch");
+    }
+    return SGF_OK;
+}
+
+// The block-convolution part of a batch (plans[k]->blk): block arguments indexed
+// like the plans' solve arguments, CTA prefixes, and the products of all plans with
+// whole addresses (in complex elements) in place of offsets.
+template <typename T>
+sgf_status batch_build_blocks(sgf_batch *bt)
+{
+    using C = typename BlkArgs<T>::C;
+    std::vector<BlkArgs<T>> args(bt->plans.size());
+    std::vector<int> index, prefix;
+    std::vector<BlkTarget> targets;
+    for (int k = 0; k < (int)bt->plans.size(); ++k) {
+        const sgf_plan *p = bt->plans[k];
+        if (!p->blk)
+            continue;
+        index.push_back(k);
+        fill_blk<T>(p, p->d_fwd, args[k]);
+        const size_t spec = reinterpret_cast<size_t>(p->spec->dev) / sizeof(C);
+        const size_t x = reinterpret_cast<size_t>(args[k].x) / sizeof(C), acc = reinterpret_cast<size_t>(args[k].acc) / sizeof(C);
+        for (BlkTarget t : p->btargets) {
+            for (auto &te : t.terms) {
+                te.k_off += spec;
+                te.x_off += x;
+            }
+            t.a_off += acc;
+            targets.push_back(t);
+        }
+    }
+    bt->blk_plans = (int)index.size();
+    if (index.empty())
+        return SGF_OK;
+    for (int k : index)
+        bt->blk_rounds = std::max(bt->blk_rounds, args[k].rounds);
+    for (int ps = 0; ps < BLK_PASSES + bt->blk_rounds; ++ps) {
+        int b = 0;
+        for (int k : index) {
+            prefix.push_back(b);
+            const int r = ps - BLK_PASSES;
+            b += r < 0 ? args[k].blocks[ps][args[k].stages] : r < args[k].rounds ? args[k].seg[r][args[k].segs[r]].blk : 0;
+        }
+        prefix.push_back(b);
+        bt->blk_blocks[ps] = b;
+        bt->launches += b > 0 ? 1 : 0;
+    }
+    std::vector<MacItem> items;
+    std::vector<MacTerm> terms;
+    std::vector<size_t> xo, ao;
+    build_mac(targets, 16 / (int)sizeof(C), items, terms, xo, ao, &bt->mac_blocks);
+    bt->mac_items = (int)items.size();
+    bt->launches++;
+    std::vector<unsigned char> blob;
+    align_push(blob, args);
+    bt->off_prefix = align_push(blob, prefix);
+    bt->off_index = align_push(blob, index);
+    bt->off_items = align_push(blob, items);
+    bt->off_terms = align_push(blob, terms);
+    bt->off_xo = align_push(blob, xo);
+    bt->off_ao = align_push(blob, ao);
+    cudaError_t e;
+    if ((e = cudaMalloc(&bt->d_blk, blob.size())) != cudaSuccess)
+        return cuda_fail(e, "cudaMalloc(batch block arguments)");
+    if ((e = upload_landed(bt->d_blk, blob.data(), blob.size())) != cudaSuccess)
+        return cuda_fail(e, "cudaMemcpy(batch block arguments)");
+    if ((e = blk_prepare<T>()) != cudaSuccess)
+        return cuda_fail(e, "block kernel attributes");
     return SGF_OK;
 }
 
@@ -1731,6 +2228,7 @@ void batch_free(sgf_batch *bt)
         cudaEventDestroy(bt->uploaded);
 
     cudaFree(bt->d_args);
+    cudaFree(bt->d_blk);
     cudaFree(bt->d_maps);
     cudaFreeHost(bt->h_args);
     cudaSetDevice(cur);
@@ -1744,12 +2242,14 @@ sgf_status batch_build(sgf_batch *bt)
     bt->args_bytes = sizeof(SolveArgs<T>) * (size_t)count;
     // groups: one per (N, path), in order of first appearance
     std::vector<int2> maps;
-    std::map<std::pair<int, bool>, int> gidx;
+    std::map<std::tuple<int, bool, bool>, int> gidx;
     std::vector<std::vector<int>> members;
     for (int k = 0; k < count; ++k) {
         const sgf_plan *p = bt->plans[k];
         bt->max_n = std::max(bt->max_n, p->N);
-        auto key = std::make_pair(p->logN, p->merged);
+        // nests whose finer patches have Case-3 outputs in a group of their own, as k_row_inv takes them
+        const bool own = p->blk || p->L == p->fo.R;
+        auto key = std::make_tuple(p->logN, p->merged, p->N >= 256 && !own);
         if (!gidx.count(key)) {
             gidx[key] = (int)bt->groups.size();
             sgf_batch::Group g;
@@ -1757,9 +2257,11 @@ sgf_status batch_build(sgf_batch *bt)
             g.merged = p->merged;
             g.tc = p->tc;
             g.sched = p->sched;
+            g.own = true;
             bt->groups.push_back(g);
             members.emplace_back();
         }
+        bt->groups[gidx[key]].own &= own;
         members[gidx[key]].push_back(k);
         bt->plan_group.push_back(gidx[key]);
     }
@@ -1867,6 +2369,9 @@ sgf_status batch_build(sgf_batch *bt)
         return cuda_fail(e, "cudaEventCreate(batch upload)");
     if ((e = cudaStreamCreateWithFlags(&bt->capture_stream, cudaStreamNonBlocking)) != cudaSuccess)
         return cuda_fail(e, "cudaStreamCreate(batch capture)");
+    const sgf_status bs = batch_build_blocks<T>(bt);
+    if (bs != SGF_OK)
+        return bs;
     SolveArgs<T> dummy{};
     for (const auto &g : bt->groups)
         if ((e = launch_pass_n<T>(PASS_PREPARE, g.logN, dummy, 0, nullptr, nullptr, g.tc)) != cudaSuccess)
@@ -2095,7 +2600,7 @@ sgf_status autotune_impl(sgf_plan *p, int reps, cudaStream_t st, double ms[SGF_A
         const sgf_schedule cand = inv_cand(c);
         if (schedule_ok(p, cand))
             s = timeit([&] { return launch_row_inv<T>(p->logN, p->L, p->fo.R, a, st, p->tc, cand.row_inv0,
-                                                      cand.inv_radix, p->tmap_inv2); },
+                                                      cand.inv_radix, p->tmap_inv2, p->blk); },
                        ms[inv_slot(c)]);
     }
     if (s == SGF_OK) {  // the fastest of the candidates that apply (and were timed)
@@ -2178,7 +2683,9 @@ template <typename T>
 sgf_status prepare_kernels_t(const sgf_plan *p)
 {
     SolveArgs<T> dummy{};
-    const cudaError_t e = launch_pass_n<T>(PASS_PREPARE, p->logN, dummy, 0, nullptr, nullptr, p->tc);
+    cudaError_t e = launch_pass_n<T>(PASS_PREPARE, p->logN, dummy, 0, nullptr, nullptr, p->tc);
+    if (e == cudaSuccess && p->blk)
+        e = blk_prepare<T>();
     return e == cudaSuccess ? SGF_OK : cuda_fail(e, "kernel attributes");
 }
 
@@ -2188,8 +2695,9 @@ sgf_status prepare_kernels(const sgf_plan *p)
 }
 
 // A validated geometry's plan: lists, recorded schedule, spectra, workspace.
+// whole_grid: no block convolutions, whatever blk_applies says (the request loop).
 sgf_status plan_create(const Forest &fo, sgf_precision precision, uint32_t flags, size_t spectra_budget,
-                       sgf_plan **out)
+                       sgf_plan **out, bool whole_grid = false)
 {
     sgf_plan *p = new sgf_plan();
     plan_init(p, fo, precision, flags);
@@ -2204,6 +2712,7 @@ sgf_status plan_create(const Forest &fo, sgf_precision precision, uint32_t flags
         s = fail(SGF_EUNSUPPORTED, "no kernel schedule applies (zero-rim potential with SGF_BF16X needs n < %d)",
                  SGF_MAX_N);
     if (s == SGF_OK) {
+        p->blk = !whole_grid && blk_applies(p);
         build_lists(p);
         s = plan_stream_layout(p);
     }
@@ -2230,21 +2739,47 @@ sgf_status plan_create(const Forest &fo, sgf_precision precision, uint32_t flags
 }
 
 sgf_status plan_estimate(const Forest &fo, sgf_precision precision, uint32_t flags, size_t *workspace_bytes,
-                         size_t *spectra_bytes, size_t *build_bytes)
+                         size_t *spectra_bytes, size_t *build_bytes, bool whole_grid = false)
 {
     sgf_plan p;
     plan_init(&p, fo, precision, flags);
     sgf_status s = build_cover(&p);
     if (s != SGF_OK)
         return s;
+    p.blk = !whole_grid && blk_applies(&p);
     build_lists(&p);
     *workspace_bytes = workspace_of(&p);
     *spectra_bytes = spectra_total(&p);
-    *build_bytes = gen_workspace_bytes(p.N);
+    *build_bytes = gen_workspace_bytes(&p);
     return SGF_OK;
 }
 
 }  // namespace
+
+namespace sgf {
+
+sgf_status nest_plan_create(const sgf_nest_desc *desc, sgf_precision precision, uint32_t flags, bool whole_grid,
+                            sgf_plan **out)
+{
+    *out = nullptr;
+    sgf_status s = validate(desc, precision);
+    if (s == SGF_OK)
+        s = check_flags(desc->levels, flags);
+    return s == SGF_OK ? plan_create(forest_of_nest(desc), precision, flags, 0, out, whole_grid) : s;
+}
+
+sgf_status nest_plan_estimate(const sgf_nest_desc *desc, sgf_precision precision, uint32_t flags, bool whole_grid,
+                              size_t *workspace_bytes, size_t *spectra_bytes, size_t *build_bytes)
+{
+    sgf_status s = validate(desc, precision);
+    if (s == SGF_OK)
+        s = check_flags(desc->levels, flags);
+    return s == SGF_OK ? plan_estimate(forest_of_nest(desc), precision, flags, workspace_bytes, spectra_bytes,
+                                       build_bytes, whole_grid)
+                       : s;
+}
+
+}  // namespace sgf
 
 extern "C" {
 
@@ -2347,6 +2882,7 @@ sgf_status sgf_plan_share_ex(const sgf_plan *src, sgf_precision precision, sgf_p
     p->spectra_budget = src->spectra_budget;  // the same resident sets as src's spectra
     sgf_status s = build_cover(p);
     if (s == SGF_OK) {
+        p->blk = src->blk;  // the sets as src's spectra store them
         build_lists(p);
         // src's schedule where it applies to this plan (its precision, its lists);
         // else the choices that always do, one pass at a time
@@ -2396,11 +2932,16 @@ sgf_status sgf_plan_stats_get(const sgf_plan *p, sgf_plan_stats *st)
     st->precision = (int)p->prec;
     st->forward_slabs = (int)p->slabs.size();
     st->outputs = (int)p->outs.size();
+    for (const auto &sg : p->stages) {
+        st->forward_slabs += sg.src_count * sg.m * sg.m;
+        st->outputs += (sg.tgt_count[0] + sg.tgt_count[1]) * sg.m * sg.m;
+    }
     st->spectra_sets = (int)p->sets.size();
     // restrictions, row_fwd, col, row_inv1 (+ row_inv for the finer patches) or one row_inv for all
     st->launches_per_solve = p->restricted + 3 + (p->L > p->fo.R && p->sched.row_inv0 != 1 ? 1 : 0) +
                              (!p->groups.empty() && p->sched.col_case3 == 0 ? 1 : 0) +  // + k_col_g
-                             (p->sums.empty() ? 0 : 1);                                  // + k_col_sum
+                             (p->sums.empty() ? 0 : 1) +                                 // + k_col_sum
+                             (p->blk ? 4 + p->fo.depth - 1 : 0);  // + the block passes
     if (p->streamed) {  // column passes: one per non-empty pass; three generator kernels per streamed set
         int passes = 0, streamed_sets = 0;
         for (int ph = 0; ph <= p->waves; ++ph)
@@ -2494,11 +3035,15 @@ sgf_status sgf_solve_host(sgf_plan *p, const void *const *sigma, void *const *fx
     // sigma always goes through the staging by a copy: the copy engine reads
     // host memory faster than the forward row pass does.  Mapped page-locked
     // output buffers are written by the inverse row pass in place, over the
-    // CPU-GPU link, which saves the device-to-host copy; others are staged.
+    // CPU-GPU link, which saves the device-to-host copy; others are staged, and
+    // so are all where the cross-level pairs add to the forces after that pass
+    // (adding would read over the link what was just written; the crop of an
+    // embedded plan writes last, whatever came before).
+    const bool adds = p->blk && p->n_log == p->N;
     bool map_x[kMaxPatches], map_y[kMaxPatches];
     for (int l = 0; l < p->L; ++l) {
-        map_x[l] = host_mapped(fx[l], lvl);
-        map_y[l] = host_mapped(fy[l], lvl);
+        map_x[l] = !adds && host_mapped(fx[l], lvl);
+        map_y[l] = !adds && host_mapped(fy[l], lvl);
     }
     if (!p->d_stage) {
         if ((e = cudaMalloc(&p->d_stage, 3 * (size_t)p->L * lvl_al)) != cudaSuccess)
@@ -2671,7 +3216,7 @@ sgf_status sgf_plan_profile_read(sgf_plan *p, sgf_kernel_times *out)
         return fail(SGF_EINVAL, "NULL argument");
     DeviceGuard g(p->device);
     std::memset(out, 0, sizeof *out);
-    const size_t per = 5;  // events per solve (mark() calls)
+    const size_t per = 6;  // events per solve (mark() calls)
     cudaError_t e;
     if (p->events_used >= per && (e = cudaEventSynchronize(p->events[p->events_used - 1])) != cudaSuccess)
         return cuda_fail(e, "cudaEventSynchronize(profile)");
@@ -2684,6 +3229,10 @@ sgf_status sgf_plan_profile_read(sgf_plan *p, sgf_kernel_times *out)
             out->ms[k] += ms;
             out->launches[k] += k == 0 ? p->restricted : 1;
         }
+        float ms = 0.f;  // the cross-level pairs count as column work: their products are its spectral sums
+        if ((e = cudaEventElapsedTime(&ms, p->events[b + 4], p->events[b + 5])) != cudaSuccess)
+            return cuda_fail(e, "cudaEventElapsedTime(profile)");
+        out->ms[2] += ms;
     }
     p->events_used = 0;
     return SGF_OK;

@@ -42,6 +42,7 @@
 //   P0 = -h Int 1/r,  Px = -h (Int u/r - u_c Int 1/r),  Py = -h (Int v/r - v_c Int 1/r),
 // h the finer cell size of the pair (the force tables are scale-free, the
 // potential grows with the cell), the slope tables again scaled by 1/m in Case 3.
+#include "sgf_block.h"
 #include "sgf_fft.cuh"
 #include "sgf_internal.h"
 
@@ -210,7 +211,37 @@ __global__ void k_gen_tables(GenSet g, int N, double *__restrict__ tables)
         tables[t * plane + at] = out[t];
 }
 
-// Rows of the P x P tables -> half spectra along x: half[t][kx 0..N][y 0..P).
+// The tables of one set of a block convolution (sgf_block.cuh), N = B cells a
+// block: for block (qx, qy) of the m x m blocks of the coarser patch, at
+// tables[t][qy m + qx][2B][2B], the convolution indices d in [-(B-1), B-1] of
+// a block and a phase, i.e. D = qB + d (Case 2, target blocks) or d - qB
+// (Case 3, source blocks) in the indexing of Cases 2 and 3 above.
+__global__ void k_gen_tables_blk(GenSet g, int B, double *__restrict__ tables)
+{
+    const int P = 2 * B, at = blockIdx.x * blockDim.x + threadIdx.x;
+    const int blk = blockIdx.y, m2 = g.m * g.m;
+    if (at >= P * P)
+        return;
+    const int py = at / P, px = at - py * P;
+    const int cas = g.cas == kBlkCase2 ? 2 : 3;
+    const AxisMap mx{cas, g.m, g.px, g.ax, B * g.m}, my{cas, g.m, g.py, g.ay, B * g.m};
+    double out[6] = {0, 0, 0, 0, 0, 0};
+    if (px != B && py != B) {
+        const int dx = px < B ? px : px - P, dy = py < B ? py : py - P;
+        const int ox = (blk % g.m) * B, oy = (blk / g.m) * B;
+        const int Dx = cas == 2 ? ox + dx : dx - ox, Dy = cas == 2 ? oy + dy : dy - oy;
+        if (spec_phi(g.kind))
+            cell_tables_phi(mx, my, Dx, Dy, cas, g.m, g.h, out);
+        else
+            cell_tables(mx, my, Dx, Dy, cas, g.m, out);
+    }
+    const int ntab = spec_tables(g.kind);
+    for (int t = 0; t < ntab; ++t)
+        tables[((size_t)t * m2 + blk) * P * P + at] = out[t];
+}
+
+// Rows of the P x P tables -> half spectra along x: half[t][kx 0..N][y 0..P)
+// (t: the tables, or for block convolutions the tables of every block).
 // Two real rows ride as one complex row; the P-point transform of a row is
 // folded into two N-point transforms: bin 2k+b = DFT_N[(x[n] + (-1)^b x[n+N]) W_P^{bn}].
 __global__ void k_gen_rows(int N, int logN, const double *__restrict__ tables,
@@ -219,7 +250,7 @@ __global__ void k_gen_rows(int N, int logN, const double *__restrict__ tables,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2 *W = reinterpret_cast<double2 *>(smem_raw);
     const int P = 2 * N, tid = threadIdx.x, nt = blockDim.x;
-    const int t = blockIdx.y, y0 = 2 * blockIdx.x;
+    const int t = blockIdx.x, y0 = 2 * blockIdx.y;
     const double *ra = tables + (size_t)t * P * P + (size_t)y0 * P;
     const double *rb = ra + P;
     for (int n = tid; n < N; n += nt) {
@@ -241,15 +272,17 @@ __global__ void k_gen_rows(int N, int logN, const double *__restrict__ tables,
 }
 
 // Columns kx of the half spectra -> the stored kernel spectra (scaled by 1/P^2).
+// blocks > 0: a set of block convolutions, table t / blocks of block t % blocks,
+// stored [block][table][kx][ky parity][ky / 2].
 template <typename T>
 __global__ void k_gen_cols(int N, int logN, const double2 *__restrict__ half, const double2 *__restrict__ tw,
-                           int kind, void *spec, size_t spec_off)
+                           int kind, int blocks, void *spec, size_t spec_off)
 {
     using C = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2 *W = reinterpret_cast<double2 *>(smem_raw);
     const int P = 2 * N, tid = threadIdx.x, nt = blockDim.x;
-    const int kx = blockIdx.x, t = blockIdx.y;
+    const int kx = blockIdx.y, t = blockIdx.x;
     const double2 *col = half + ((size_t)t * (N + 1) + kx) * P;
     for (int n = tid; n < N; n += nt) {
         const double2 lo = col[n], hi = col[n + N];
@@ -259,7 +292,16 @@ __global__ void k_gen_cols(int N, int logN, const double2 *__restrict__ half, co
     __syncthreads();
     block_fft<double2, false>(W, N, logN, 2, tw);
     const double scale = 1.0 / ((double)P * (double)P);
-    if (spec_quarter(kind) || kind == SPEC_MERGED || kind == SPEC_MERGED_PHI) {
+    if (blocks > 0) {
+        const int tab = t / blocks, blk = t - tab * blocks, nt_all = gridDim.x / blocks;
+        C *dst = reinterpret_cast<C *>(spec) + spec_off + (((size_t)blk * nt_all + tab) * (N + 1) + kx) * P;
+        for (int i = tid; i < P; i += nt) {  // the transform's halves are the ky parities
+            C v;
+            v.x = (T)(W[i].x * scale);
+            v.y = (T)(W[i].y * scale);
+            dst[i] = v;
+        }
+    } else if (spec_quarter(kind) || kind == SPEC_MERGED || kind == SPEC_MERGED_PHI) {
         // K0x and K0y (tables 0, 3) are odd in one axis: purely imaginary; merged Gx, Gy
         // too; of the potential tables Px and Py (1, 2), while P0 is real
         const int QS = quarter_stride(N), HQ = quarter_half(N);
@@ -310,6 +352,24 @@ cudaError_t launch_gen_set(const GenSet &g, int N, int logN, const double2 *tw64
                            double *work_tables, double2 *work_half, cudaStream_t st)
 {
     const int P = 2 * N;
+    if (gen_blk(g)) {
+        const int B = N / g.m, m2 = g.m * g.m, nt = spec_tables(g.kind);
+        const double2 *twb = tw64 + 2 * P - 2 * P / g.m;  // W_2B^k, after the larger tables
+        k_gen_tables_blk<<<dim3((4 * B * B + 255) / 256, m2), 256, 0, st>>>(g, B, work_tables);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess)
+            return e;
+        int logB = 0;
+        while ((1 << logB) < B)
+            ++logB;
+        const size_t smem = 2 * (size_t)B * sizeof(double2);
+        k_gen_rows<<<dim3(nt * m2, B), gen_threads(B), smem, st>>>(B, logB, work_tables, work_half, twb);
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            return e;
+        k_gen_cols<T><<<dim3(nt * m2, B + 1), gen_threads(B), smem, st>>>(B, logB, work_half, twb, g.kind, m2, spec,
+                                                                        g.spec_off);
+        return cudaGetLastError();
+    }
     {
         const int bs = 256;
         dim3 grid((P + bs - 1) / bs, P);
@@ -320,10 +380,10 @@ cudaError_t launch_gen_set(const GenSet &g, int N, int logN, const double2 *tw64
         return e;
     const size_t smem = 2 * (size_t)N * sizeof(double2);
     const int ntab = spec_tables(g.kind);
-    k_gen_rows<<<dim3(P / 2, ntab), gen_threads(N), smem, st>>>(N, logN, work_tables, work_half, tw64);
+    k_gen_rows<<<dim3(ntab, P / 2), gen_threads(N), smem, st>>>(N, logN, work_tables, work_half, tw64);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    k_gen_cols<T><<<dim3(N + 1, ntab), gen_threads(N), smem, st>>>(N, logN, work_half, tw64, g.kind, spec,
+    k_gen_cols<T><<<dim3(ntab, N + 1), gen_threads(N), smem, st>>>(N, logN, work_half, tw64, g.kind, 0, spec,
                                                                      g.spec_off);
     return cudaGetLastError();
 }

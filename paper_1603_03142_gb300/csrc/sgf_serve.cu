@@ -35,6 +35,7 @@ struct Pending {
     std::string key;   // slot key: spectra key + precision
     std::string skey;  // spectra key
     size_t ws = 0, spectra = 0, build = 0, io = 0;  // bytes (sgf_plan_estimate; io = 3 L n^2 elements)
+    bool whole_grid = false;  // plans without block convolutions
     size_t stream_budget = 0;  // SGF_SERVER_STREAM: the spectra budget of this shape's plans, else 0
     double t_submit = 0;
 };
@@ -206,7 +207,7 @@ sgf_status slot_create(sgf_server *sv, const Pending &p, Slot **out)
                       : fail(SGF_EINVAL, "resident shape without a slot");
         } else if (rc == SGF_OK) {
             rc = p.stream_budget ? sgf_plan_create(&p.r.desc, p.r.precision, p.stream_budget, &s->plan)
-                                 : sgf_plan_create_ex(&p.r.desc, p.r.precision, p.r.plan_flags, &s->plan);
+                                 : nest_plan_create(&p.r.desc, p.r.precision, p.r.plan_flags, p.whole_grid, &s->plan);
         }
         // the kernel schedule of this slot key: tuned once per server (on the slot's own
         // stream, while the other slots keep running), then reused
@@ -340,7 +341,10 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
         return fail(SGF_EINVAL, "NULL argument");
     Pending p;
     p.r = *r;
-    sgf_status rc = sgf_plan_estimate(&r->desc, r->precision, r->plan_flags, &p.ws, &p.spectra, &p.build);
+    // FP32 and SGF_BF16X requests of a shape share its spectra: from four levels on, where
+    // SGF_BF16X plans keep the whole-grid passes, every request of the shape does
+    p.whole_grid = r->desc.levels >= 4;
+    sgf_status rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, p.whole_grid, &p.ws, &p.spectra, &p.build);
     if (rc != SGF_OK)
         return rc;
     if (r->plan_flags & SGF_PLAN_POTENTIAL)
@@ -354,6 +358,14 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
     p.io = 3 * (size_t)L * align256(lvl);
     p.skey = spectra_key(*r);
     p.key = p.skey + "/p" + std::to_string((int)r->precision);
+    if (!p.whole_grid && p.ws + p.io + p.spectra + p.build > sv->cfg.hbm_budget) {
+        // the block convolutions' spectra are up to 2% larger than the whole-grid passes': a shape
+        // that fits only as those is served so
+        p.whole_grid = true;
+        rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, true, &p.ws, &p.spectra, &p.build);
+        if (rc != SGF_OK)
+            return rc;
+    }
     if (sv->cfg.max_shape_bytes && p.spectra + p.build > sv->cfg.max_shape_bytes &&
         (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0 && p.build < sv->cfg.max_shape_bytes) {
         // served by plans over a spectra budget: resident sets and a window within the budget,

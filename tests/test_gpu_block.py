@@ -1,0 +1,156 @@
+"""Cross-level pairs as block convolutions (nests and forests of N >= 256): the
+coarser patch cut into m x m blocks of B = N/m cells, every phase and block pair a
+convolution zero-padded to 2B (Sec. 2.2, Eqs. eqnbmnn and eqnbnmn).  Against the
+direct-sum oracle on sampled cells, within the bounds of tests/_gpu.py, at the
+edges of the block sizes (B = 16 ... 2048), on odd offsets, embedded sizes,
+forests (several sources per target) and potentials; the no-allocation solve and
+batches (kernel spectra shared by up to four right-hand sides) bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1603_03142_gb300 import workloads as W
+from tests._gpu import run_gpu, sgf, tol, torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    return sgf()
+
+
+def _sigma(geom, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    return [rng.uniform(0.2, 1.5, (geom.n, geom.n)) for _ in range(geom.levels)]
+
+
+def _sample(geom, per_patch, seed):
+    """Seeded uncovered cells of every patch, with the patch's corners and edges' midpoints."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    n, lv, ii, jj = geom.n, [], [], []
+    edge = {(0, 0), (0, n - 1), (n - 1, 0), (n - 1, n - 1), (n // 2, 0), (0, n // 2), (n // 2, n - 1), (n - 1, n // 2)}
+    for p in range(geom.levels):
+        cov = geom.covered_mask(p)
+        free = np.argwhere(~cov)
+        pick = [tuple(x) for x in free[rng.choice(len(free), size=per_patch, replace=False)]]
+        pick += [c for c in edge if not cov[c]][:max(0, per_patch // 2)]
+        for j, i in pick:
+            lv.append(p), jj.append(j), ii.append(i)
+    return np.array(lv), np.array(ii), np.array(jj)
+
+
+def _worst(geom, got, ref, samp):
+    lv, ii, jj = samp
+    worst = 0.0
+    for p in range(geom.levels):
+        m = lv == p
+        scale = max(np.abs(r[m]).max() for r in ref)
+        worst = max(worst, max(np.abs(g[p][jj[m], ii[m]] - r[m]).max() for g, r in zip(got, ref)) / scale)
+    return worst
+
+
+NESTS = {
+    "256x2_corner": (W.Nest(n=256, levels=2, off=[(0, 0), (0, 128)]), ("fp32", "bf16x")),
+    "256x3_odd": (W.Nest(n=256, levels=3, off=[(0, 0), (37, 90), (101, 3)]), ("fp32", "bf16x")),
+    "256x5": (W.Nest(n=256, levels=5, off=[(0, 0), (64, 65), (63, 7), (128, 64), (31, 33)]), ("fp32",)),
+    "300x3_embedded": (W.Nest(n=300, levels=3, off=[(0, 0), (75, 11), (150, 80)]), ("fp32",)),
+    "1024x4": (W.Nest(n=1024, levels=4, off=[(0, 0), (255, 256), (301, 4), (256, 511)]), ("fp32",)),
+    "2048x2": (W.Nest(n=2048, levels=2, off=[(0, 0), (513, 700)]), ("fp32",)),
+    "4096x2": (W.Nest(n=4096, levels=2, off=[(0, 0), (1025, 1000)]), ("fp32",)),
+    "two_patches256": (W.two_patch_forest(256), ("fp32",)),
+    "example4_256": (W.example4_forest(256), ("fp32",)),
+}
+
+
+@pytest.mark.parametrize("name,prec", [(k, p) for k, (_, ps) in NESTS.items() for p in ps])
+def test_block_pairs_against_oracle(lib, name, prec):
+    geom = NESTS[name][0]
+    sigma = _sigma(geom, 3)
+    plan = lib.Plan(geom, prec)
+    gx, gy = run_gpu(plan, sigma)
+    plan.check()
+    samp = _sample(geom, 4 if geom.n >= 2048 else 16, 5)
+    ox, oy = oracle.force_at(geom, sigma, *samp)
+    assert _worst(geom, (gx, gy), (ox, oy), samp) <= tol(prec, geom.n)
+
+
+@pytest.mark.parametrize("name", ["256x2_corner", "256x3_odd", "256x5", "300x3_embedded"])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_block_pairs_equal_whole_grid_pairs(lib, name, prec):
+    """A plan over its spectra budget runs the whole-grid passes on the same FP64 tables: the
+    same sums in another order (256 ulps, the bound of the budget tests).  In FP64 this says
+    more than the oracle: away from m = 1 both paths share the tables' own error."""
+    geom = NESTS[name][0]
+    sigma = _sigma(geom, 11)
+    plan = lib.Plan(geom, prec)
+    whole = lib.Plan(geom, prec, spectra_budget=plan.stats()["spectra_bytes"] // 2)
+    assert whole.stats()["spectra_sets_streamed"] > 0
+    a, b = run_gpu(plan, sigma), run_gpu(whole, sigma)
+    eps = np.finfo(np.float64 if prec == "fp64" else np.float32).eps
+    for l in range(geom.levels):
+        scale = max(np.abs(b[0][l]).max(), np.abs(b[1][l]).max())
+        d = max(np.abs(a[c][l] - b[c][l]).max() for c in range(2))
+        assert d <= 256 * eps * scale, (l, d / scale)
+
+
+@pytest.mark.parametrize("prec", ["fp32"])
+def test_block_potential_against_oracle(lib, prec):
+    geom = NESTS["256x3_odd"][0]
+    sigma = _sigma(geom, 4)
+    plan = lib.Plan(geom, prec, potential=True)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    phi = plan.solve_potential([torch.from_numpy(s).to(device="cuda", dtype=dt) for s in sigma])
+    torch.cuda.synchronize()
+    samp = _sample(geom, 16, 6)
+    ref = oracle.potential_at(geom, sigma, *samp)
+    assert _worst(geom, ([p.double().cpu().numpy() for p in phi],), (ref,), samp) <= tol(prec, geom.n)
+
+
+def test_block_noalloc_is_bitwise_the_solve(lib):
+    for geom in (W.Nest(n=256, levels=3, off=[(0, 0), (64, 20), (33, 64)]), W.two_patch_forest(256)):
+        plan = lib.Plan(geom, "fp32")
+        sig = [torch.from_numpy(s).float().cuda() for s in _sigma(geom, 8)]
+        fx, fy = plan.solve(sig)
+        gx, gy = [torch.empty_like(s) for s in sig], [torch.empty_like(s) for s in sig]
+        plan.solve_noalloc_ptrs([s.data_ptr() for s in sig], [t.data_ptr() for t in gx], [t.data_ptr() for t in gy])
+        torch.cuda.synchronize()
+        for l in range(geom.levels):
+            assert torch.equal(fx[l], gx[l]) and torch.equal(fy[l], gy[l])
+
+
+@pytest.mark.parametrize("count", [1, 3, 6])
+def test_block_batch_is_bitwise_the_single_solves(lib, count):
+    """`count` centred nests on shared spectra (their level pairs share sets too), one nest of
+    another shape, one deep nest on whole-grid passes (B would be 8), one uniform grid."""
+    base = lib.Plan(W.centred_nest(256, 3), "fp32")
+    plans = [base] + [base.share() for _ in range(count - 1)]
+    plans += [lib.Plan(W.centred_nest(512, 2, centre=(0.3, 0.1)), "fp32"), lib.Plan(W.centred_nest(256, 6), "fp32"),
+              lib.Plan(W.Nest(n=256), "fp32")]
+    sig = [[torch.from_numpy(s).float().cuda() for s in _sigma(p.nest, 20 + k)] for k, p in enumerate(plans)]
+    single = [p.solve(s) for p, s in zip(plans, sig)]
+    torch.cuda.synchronize()
+    batch = lib.Batch(plans)
+    fx, fy = [[torch.empty_like(s) for s in lst] for lst in sig], [[torch.empty_like(s) for s in lst] for lst in sig]
+    for _ in range(2):
+        batch.solve(sig, fx, fy)
+    torch.cuda.synchronize()
+    for k, p in enumerate(plans):
+        for l in range(p.levels):
+            assert torch.equal(fx[k][l], single[k][0][l]) and torch.equal(fy[k][l], single[k][1][l]), (k, l)
+
+
+def test_bf16x_depths_and_shared_spectra(lib):
+    """SGF_BF16X of four levels keeps the whole-grid passes; a plan shared from FP32 takes the
+    spectra as they are stored; both within the precision's bound of FP32."""
+    for levels in (3, 4):
+        nest = W.centred_nest(256, levels)
+        sigma = _sigma(nest, 30)
+        p32 = lib.Plan(nest, "fp32")
+        ref = run_gpu(p32, sigma)
+        for p in (lib.Plan(nest, "bf16x"), p32.share("bf16x"), lib.Plan(nest, "bf16x").share("fp32")):
+            got = run_gpu(p, sigma)
+            p.check()
+            for l in range(levels):
+                scale = max(np.abs(ref[0][l]).max(), np.abs(ref[1][l]).max())
+                assert max(np.abs(got[c][l] - ref[c][l]).max() for c in range(2)) <= tol("bf16x", 256) * scale

@@ -13,9 +13,9 @@
 // (m^4 blocks of (B + 1) x 2B, six tables) are as many values as m^2 sets of
 // (N + 1) x 2N, read once per solve: the stage is bound by streaming them.
 //
-// Measured (FP32, GB300; whole-grid passes -> this): 1024^2 3 levels 2027 -> 1375 us,
-// 2048^2 2 levels 2208 -> 1911, 256^2 3 levels 278 -> 175, six 256^2 tiles and
-// two refined patches 593 -> 330, 20 nests of 128 ... 1024 cells 3362 -> 1990.
+// Measured (FP32, GB300; whole-grid passes -> this): 1024^2 3 levels 2027 -> 1331 us,
+// 2048^2 2 levels 2208 -> 1832, 256^2 3 levels 278 -> 167, six 256^2 tiles and
+// two refined patches 593 -> 327, 20 nests of 128 ... 1024 cells 3362 -> 1936.
 //
 // Passes of a solve, each one launch over every stage (one stage per m):
 //   k_blk_rows   cells -> (sigma, dx, dy) of a source unit (phase or block),
@@ -105,6 +105,19 @@ __device__ __forceinline__ bool blk_covered(const SolveArgs<T> &a, int patch, in
 // Cell of element (r, c) of a unit: kind 0 = phase (every m-th cell), 1 = block of B x B cells.
 __device__ __forceinline__ int blk_cell(int kind, int m, int B, int u, int r) { return kind == 0 ? m * r + u : u * B + r; }
 
+// Element e of a CTA's cells in the order of the patch's rows: its sequence and its
+// column there (2^lmm units of a row pair: phases interleave, blocks follow one another).
+struct BlkElem {
+    int gg, c;
+};
+template <int LOGB>
+__device__ __forceinline__ BlkElem blk_elem(int e, int lmm, int kind)
+{
+    const int w = e & ((1 << (LOGB + lmm)) - 1), pr = e >> (LOGB + lmm);
+    const int ux = kind == 0 ? w & ((1 << lmm) - 1) : w >> LOGB;
+    return BlkElem{(pr << lmm) + ux, kind == 0 ? w >> lmm : w & ((1 << LOGB) - 1)};
+}
+
 // ------------------------------------------------------------------ rows
 // The sequences of a CTA are the m units of one row pair (their columns together
 // are the pair's whole rows; N = 4096: half of them), for 2048/N row pairs: a
@@ -157,34 +170,47 @@ __device__ __forceinline__ void blk_rows_body(const SolveArgs<T> &a, const BlkAr
 #pragma unroll 1
     for (int f = f0; f < f0 + fields; ++f) {
         // field f of the CTA's cells, the two rows of a pair as one complex value, element c of
-        // sequence gg at sbuf[2 gg SP + pad16(c)]; in the order of the patch's rows, so that loads coalesce
-#pragma unroll 2
-        for (int e = t; e < G * B; e += kBlkThreads) {
-            const int w = e & (B * (1 << lmm) - 1), pr = e >> (LOGB + lmm);
-            const int uxl = un.kind == 0 ? w & ((1 << lmm) - 1) : w >> LOGB;
-            const int c = un.kind == 0 ? w >> lmm : w & (B - 1);
-            const int gg = (pr << lmm) + uxl;
-            const BlkSeq &q = seq[gg];
-            const int i = q.i0 + st * c;
-            T x[2] = {T(0), T(0)};
-            if (i < nl) {
+        // sequence gg at sbuf[2 gg SP + pad16(c)]; in the order of the patch's rows, so that loads
+        // coalesce, and loaded whether used or not (at clamped cells), so that those of four
+        // elements are in flight at once (1024^2 3 levels: 134 -> 121 us)
+#pragma unroll 1
+        for (int e0 = t; e0 < G * B; e0 += 4 * kBlkThreads) {
+            T hi[4][2], lo[4][2];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const BlkElem el = blk_elem<LOGB>(e0 + w * kBlkThreads, lmm, un.kind);
+                const BlkSeq &q = seq[el.gg];
+                const int i = min(q.i0 + st * el.c, nl - 1);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int jj = q.j[h];
-                    if (jj >= nl || blk_covered(a, un.patch, jj, i, q.xa[h], q.xb[h]))
-                        continue;
+                    const int jj = min(q.j[h], nl - 1);
                     const T *r = src + (size_t)jj * N + i;
-                    if (f == 0) {
-                        x[h] = __ldg(r);
-                    } else {  // central difference, one-sided on the patch's first and last cell
-                        const int at = f == 1 ? i : jj, step = f == 1 ? 1 : N;
-                        const bool lo = at > 0, hi = at < nl - 1;
-                        const T d = __ldg(hi ? r + step : r) - __ldg(lo ? r - step : r);
-                        x[h] = lo && hi ? T(0.5) * d : d;
-                    }
+                    // central difference, one-sided on the patch's first and last cell
+                    const int at = f == 1 ? i : jj, step = f == 0 ? 0 : f == 1 ? 1 : N;
+                    hi[w][h] = __ldg(at < nl - 1 ? r + step : r);
+                    lo[w][h] = f == 0 ? T(0) : __ldg(at > 0 ? r - step : r);
                 }
             }
-            sbuf[2 * gg * SP + pad16(c)] = hmk<C>(x[0], x[1]);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const BlkElem el = blk_elem<LOGB>(e0 + w * kBlkThreads, lmm, un.kind);
+                const BlkSeq &q = seq[el.gg];
+                const int i = q.i0 + st * el.c;
+                T x[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int jj = q.j[h], at = f == 1 ? i : jj;
+                    const bool live = i < nl && jj < nl && !blk_covered(a, un.patch, jj, i, q.xa[h], q.xb[h]);
+                    T d = hi[w][h];
+                    if (f != 0) {
+                        d -= lo[w][h];
+                        if (at > 0 && at < nl - 1)
+                            d *= T(0.5);
+                    }
+                    x[h] = live ? d : T(0);
+                }
+                sbuf[2 * el.gg * SP + pad16(el.c)] = hmk<C>(x[0], x[1]);
+            }
         }
         __syncthreads();
         C v[1][16];
@@ -327,6 +353,9 @@ __device__ __forceinline__ void blk_icols_body(const BlkArgs<T> &k, const BlkSta
 // 1, phases of the finer patch).  The sequences of a CTA are consecutive row
 // pairs of a block, or the m phases of a row pair (as in the forward row pass), so
 // that the phases interleave in shared memory and runs of whole rows are added.
+// The bins come in as asynchronous copies, all in flight at once: loaded into
+// registers one after the other their latency was most of the pass (1024^2 3
+// levels: two launches of 65 us, now 51; 2048^2 2 levels 167 -> 113).
 template <typename T, int LOGB>
 __device__ __forceinline__ void blk_irows_body(const SolveArgs<T> &a, const BlkArgs<T> &k, const BlkStage &s,
                                                int target, int lb, unsigned char *smem)
@@ -380,9 +409,22 @@ __device__ __forceinline__ void blk_irows_body(const SolveArgs<T> &a, const BlkA
     };
     T *ox = a.fx[patch], *oy = nc == 2 ? a.fy[patch] : nullptr;
     const int st = kind == 0 ? 1 : m;
-    // runs of cells that lie one after the other (all phases of a row pair in this CTA): their
-    // forces are copied in behind the transforms
-    const bool whole = kind == 0 || m <= G;
+    const bool whole = kind == 0 || m <= G;  // runs of cells one after the other (all phases of a row pair)
+    for (int e = t; e < G * (B + 1); e += kBlkThreads) {
+        const int pr = e & (pairs - 1), r = e >> lp;
+        const int uxl = r / (B + 1), kx = r - uxl * (B + 1);
+        const int gg = (pr << lmm) + uxl;
+        const long long off = seq[gg].off;
+        if (off >= 0) {
+            C *dst = reinterpret_cast<C *>(stg + (gg * 2 + (kx & 1)) * HALF + (kx >> 1));
+            const C *col = k.acc + off + (size_t)kx * (2 * B);
+            cp16(dst, col);
+            if constexpr (sizeof(T) == 8)
+                cp16(dst + 1, col + 1);
+        }
+    }
+    cp_commit();
+    // the forces the CTA adds to: copied in behind the transforms where they lie one after the other
     if (whole) {
         constexpr int V = 16 / (int)sizeof(T);
         for (int e = V * t; e < kBlkCells; e += V * kBlkThreads) {
@@ -393,16 +435,7 @@ __device__ __forceinline__ void blk_irows_body(const SolveArgs<T> &a, const BlkA
         }
     }
     cp_commit();
-    for (int e = t; e < G * (B + 1); e += kBlkThreads) {
-        const int pr = e & (pairs - 1), r = e >> lp;
-        const int uxl = r / (B + 1), kx = r - uxl * (B + 1);
-        const int gg = (pr << lmm) + uxl;
-        const long long off = seq[gg].off;
-        if (off >= 0)
-            stg[(gg * 2 + (kx & 1)) * HALF + (kx >> 1)] =
-                *reinterpret_cast<const C2 *>(k.acc + off + (size_t)kx * (2 * B));
-    }
-    cp_wait<1>();  // the twiddles; the forces may still be on their way
+    cp_wait<1>();  // twiddles and bins; the forces may still be on their way
     __syncthreads();
     const int g = t / (2 * Q), b = (t / Q) & 1, j = t & (Q - 1);
     const bool valid = seq[g].off >= 0;

@@ -564,9 +564,12 @@ size_t blk_set_elems(const sgf_plan *p, const GenSet &g)
     return (size_t)spec_tables(g.kind) * g.m * g.m * blk_freqs(p->logN - ilog2(g.m));
 }
 
-// Where the block transforms apply: nests (forests) of N >= 256, and blocks of at least 16 cells
-// (the smallest transform) at the plan's depth.  Below 256 the whole-grid
-// passes take fewer launches for transforms that are launch-bound anyway.
+// Where the block transforms apply: nests (forests) of N >= 256 with blocks of at
+// least 16 cells (the smallest transform) at the plan's depth.  Below 256 the
+// whole-grid passes take fewer launches for transforms that are launch-bound
+// anyway, and so they do for FP32 potentials of a few patches on two levels at 256
+// (us per solve, whole-grid / block: 65.5 / 73.8; forces 76.8 / 79.1, but blocks save
+// a batch more; eight patches 556 / 327; three levels 258 / 147; FP64 forces 528 / 434).
 // SGF_BF16X plans of four levels and more stay with the whole-grid passes: the
 // block transforms run in FP32, and from that depth on the split-BF16 rounding
 // they leave out moves the finest level's forces by more than 2e-5 (2-norm;
@@ -574,7 +577,7 @@ size_t blk_set_elems(const sgf_plan *p, const GenSet &g)
 bool blk_applies(const sgf_plan *p)
 {
     return !p->merged && p->fo.depth > 1 && p->N >= 256 && (p->N >> (p->fo.depth - 1)) >= 16 &&
-           !(p->tc && p->fo.depth > 3);
+           (p->N > 256 || p->fo.depth > 2 || p->fo.K > 3 || !p->pot || p->esize == 8) && !(p->tc && p->fo.depth > 3);
 }
 
 // Twiddle area of the B-point block transforms within Spectra::twb (complex entries).
@@ -1455,7 +1458,7 @@ size_t gen_workspace_bytes(const sgf_plan *p)
 }
 
 // Twiddle area (tw_layout) of the transforms of N = 2^logN points, from W_Q^k, k < Q = re.size()
-// (a multiple of 2N): stage tables W_{R Ns}^{r k}, then W_P^j, then W_32^u (P = 2N).
+// (a multiple of 2N): stage tables W_{R Ns}^{r k}, then W_P^j, then W_32^u, then W_N^i (P = 2N).
 template <typename C>
 std::vector<C> solve_twiddles(int logN, const std::vector<double> &re, const std::vector<double> &im)
 {
@@ -1494,6 +1497,8 @@ std::vector<C> solve_twiddles(int logN, const std::vector<double> &re, const std
         put(tl.base + jj, jj);
     for (int u = 0; u < 16; ++u)
         put(tl.w32 + u, (long)u * (P / 32));
+    for (int i = 0; N <= kSlot4Max && i < N; ++i)
+        put(tl.full + i, 2L * i);
     return tw;
 }
 

@@ -24,6 +24,7 @@
 #pragma once
 #include <cstring>
 #include "sgf_fft.cuh"
+#include "sgf_internal.h"
 #ifdef __CUDACC__
 #include "sgf_tc.cuh"
 #endif
@@ -513,6 +514,87 @@ __device__ __forceinline__ void fft_ct(C (*v)[16], C *sbuf, int SP, int j, bool 
                                        TcCtx *tc = nullptr, int half = 0)
 {
     fft_stages<C, INV, LOGN, B, 0, TC, HB>(v, sbuf, SP, j, active, tw, tc, half);
+}
+#endif
+
+#ifdef __CUDACC__
+// ---------------------------------------------------------------------------
+// Small transforms (N = 16 .. 256): four values per thread, radix-4 stages and one
+// closing radix-2 stage when log2(N) is odd.  A slot (j, j < N/4) holds elements
+// j + u N/4, so a sequence takes N/4 lanes instead of N/16: a 64-point transform
+// fills half a warp with about 90 operations a thread where the radix-16 engine has
+// 4 lanes work through 400.  These sizes are bound by that chain: in FP64, where an
+// SM issues a warp instruction about every 16 cycles however few of its lanes are at
+// work, and in FP32, where a solve is three kernels of a few warps per SM.
+// us per solve, radix-16 slots -> these (one level; N = 64, 128, 256):
+// FP64 141 -> 47, 154 -> 55, 180 -> 100; FP32 28.6 -> 18.6, 28.7 -> 18.8,
+// 30.3 -> 23.6.  From 512 on the sequences fill their warps with 16 values a thread.
+// Stage twiddles W_{R Ns}^{r k} = W_N^{r k N / (R Ns)} come from the table W_N^i of
+// the twiddle area.
+template <typename C, bool INV, int LOGN, int B, int ST, int HB>
+__device__ __forceinline__ void fft4_stages(C (*v)[4], C *sbuf, int SP, int j, bool active, const C *wn, int half)
+{
+    constexpr int N = 1 << LOGN, Q = N / 4, S4 = LOGN / 2, NST = S4 + (LOGN & 1), NS = 1 << (2 * ST);
+    if constexpr (ST < NST) {
+        constexpr int R = ST < S4 ? 4 : 2;
+        if constexpr (ST > 0) {
+            xsync<HB>(half);  // previous stage's stores are visible
+            if (active) {
+#pragma unroll
+                for (int bb = 0; bb < B; ++bb)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        v[bb][u] = sbuf[bb * SP + pad16(j + u * Q)];
+            }
+        }
+        if (active) {
+#pragma unroll
+            for (int bb = 0; bb < B; ++bb) {
+                if constexpr (R == 4) {
+                    if constexpr (NS > 1) {
+                        const int k = j & (NS - 1);
+#pragma unroll
+                        for (int r = 1; r < 4; ++r) {
+                            const C w = wn[r * k * (N / (4 * NS))];
+                            v[bb][r] = INV ? hmulc(v[bb][r], w) : hmul(v[bb][r], w);
+                        }
+                    }
+                    hdft4<C, INV>(v[bb][0], v[bb][1], v[bb][2], v[bb][3]);
+                } else {  // butterflies (0, 2) and (1, 3) of the slot, at j and j + N/4; NS = N/2
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const C w = wn[j + q * Q];
+                        const C x = v[bb][q], y = INV ? hmulc(v[bb][q + 2], w) : hmul(v[bb][q + 2], w);
+                        v[bb][q] = badd(x, y);
+                        v[bb][q + 2] = bsub(x, y);
+                    }
+                }
+            }
+        }
+        if constexpr (ST + 1 < NST) {
+            xsync<HB>(half);  // every thread has read this stage's inputs
+            if (active) {
+                const int k = j & (NS - 1);
+                const int base = (j - k) * 4 + k;
+#pragma unroll
+                for (int bb = 0; bb < B; ++bb)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        sbuf[bb * SP + pad16(base + r * NS)] = v[bb][r];
+            }
+        }
+        fft4_stages<C, INV, LOGN, B, ST + 1, HB>(v, sbuf, SP, j, active, wn, half);
+    }
+}
+
+// fft_ct with slots of four values (chosen by the array's type).
+template <typename C, bool INV, int LOGN, int B = 1, bool TC = false, int HB = 0>
+__device__ __forceinline__ void fft_ct(C (*v)[4], C *sbuf, int SP, int j, bool active, const C *tw,
+                                       TcCtx * = nullptr, int half = 0)
+{
+    static_assert(!TC && (1 << LOGN) <= kSlot4Max, "FP32 / FP64 engine of small transforms");
+    constexpr int FULL = tw_layout(F16<LOGN>::twlen, 1 << LOGN).full;
+    fft4_stages<C, INV, LOGN, B, 0, HB>(v, sbuf, SP, j, active, tw + FULL, half);
 }
 #endif
 

@@ -209,17 +209,20 @@ static_assert(sizeof(SolveArgs<double>) + 32 <= 4096, "SolveArgs exceeds the ker
 //   [0, twlen)            radix-16 engine stage tables (Fft16Plan::twoff), W_{R Ns}^{r k}
 //   [twlen, twlen + N/16) W_P^j, j < N/16 (P = 2N)
 //   [.. + 16)             W_32^u, u < 16
+//   [.. + N)              W_N^i, N <= kSlot4Max only (the radix-4 engine's stage twiddles)
 // so that the twist W_P^n of element n = j + u N/16 is W_P^j W_32^u.
+constexpr int kSlot4Max = 256;  // largest transform of the engine with four values per thread
 struct TwLayout {
-    int twlen, base, w32, entries;
+    int twlen, base, w32, full, entries;
 };
-inline __host__ __device__ TwLayout tw_layout(int twlen, int N)
+inline constexpr __host__ __device__ TwLayout tw_layout(int twlen, int N)
 {
-    TwLayout t;
+    TwLayout t{};
     t.twlen = twlen;
     t.base = twlen;
     t.w32 = twlen + N / 16;
-    t.entries = (t.w32 + 16 + 1) & ~1;
+    t.full = t.w32 + 16;
+    t.entries = (t.full + (N <= kSlot4Max ? N : 0) + 1) & ~1;
     return t;
 }
 

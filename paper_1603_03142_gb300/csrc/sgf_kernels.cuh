@@ -97,6 +97,17 @@ __device__ __forceinline__ C twist(const C *tw, const TwLayout &tl, int j, int u
     return hmul(tw[tl.base + j], hmk<C>((T)kW32c[u], (T)-kW32s[u]));
 }
 
+// The same for the slots of four values (small transforms, see fft4_stages): n = j + u N/4,
+// j = j' + w N/16, so W_P^n = W_P^j' W_32^{w + 4 u}, both from the twiddle area.
+template <typename C, int V>
+__device__ __forceinline__ C twist_v(const C *tw, const TwLayout &tl, int N, int j, int u)
+{
+    if constexpr (V == 16)
+        return twist(tw, tl, j, u);
+    else
+        return hmul(tw[tl.base + (j & (N / 16 - 1))], tw[tl.w32 + j / (N / 16) + 4 * u]);
+}
+
 // Sequence stride (complex) of a column-pass exchange buffer: N + N/16 rounded
 // up so the next buffer starts on a 16-byte boundary.
 template <typename C>
@@ -117,14 +128,16 @@ __device__ __forceinline__ bool covered(const SolveArgs<T> &a, int s, int j, int
     return false;
 }
 
-template <int LOGN>
+// Values per thread (a "slot"): 16, or 4 for transforms of up to kSlot4Max points (FP32 and
+// FP64 engines), where 16 would leave 1 to 16 lanes of a warp at work: see fft4_stages.
+template <int LOGN, bool TC = false>
 struct KShape {
-    static constexpr int N = 1 << LOGN, Q = N >> 4;
+    static constexpr int N = 1 << LOGN, V = !TC && N <= kSlot4Max ? 4 : 16, Q = N / V;
     static constexpr int ROW_THREADS = 2 * Q < 32 ? 32 : 2 * Q;  // both parity halves
     static constexpr int COL_THREADS = Q < 32 ? 32 : Q;          // one parity half
-    static constexpr int SP_ROW = N + Q + 8;  // pad puts the two halves 16 banks apart for the unpack
+    static constexpr int SP_ROW = N + N / 16 + 8;  // pad puts the two halves 16 banks apart for the unpack
     // threads per parity half for the half barriers of the row kernels (0: whole-block barriers)
-    static constexpr int HB_ROW = Q >= 32 ? Q : 0;
+    static constexpr int HB_ROW = V == 16 && Q >= 32 ? Q : 0;
 };
 
 // Tensor-core tiles (SGF_BF16X) issued per round, i.e. A-tile buffers in shared
@@ -160,17 +173,17 @@ __host__ __device__ constexpr int tc_round(int logn, int tiles, int kind)
 // twiddles and the exchange buffers only (two CTAs per SM in FP32).
 // Shared memory: twiddle area | sbuf[2 SP_ROW] (first the staged rows).
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !TC ? 2 : 1)
+__global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS, sizeof(T) == 4 && !TC ? 2 : 1)
     k_row_fwd(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.x] : make_int2(0, (int)blockIdx.x);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
     using C2 = typename Cx<T>::C2;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, SP = K::SP_ROW;
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::ROW_THREADS, 1);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::ROW_THREADS, 1);
     constexpr int TCR = tc_round(LOGN, TCT, KK_ROW_FWD);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -206,10 +219,10 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     cp_wait<0>();
     __syncthreads();
-    C v[1][16];
+    C v[1][K::V];
     if (active) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < K::V; ++u) {
             const int c = j + u * Q;
             T fv[2] = {T(0), T(0)};
             if (c < rows) {
@@ -234,7 +247,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
             }
             C z = hmk<C>(fv[0], fv[1]);
             if (b)
-                z = hmul(z, twist(tw, tl, j, u));
+                z = hmul(z, twist_v<C, K::V>(tw, tl, N, j, u));
             v[0][u] = z;
         }
     }
@@ -244,7 +257,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
     __syncthreads();
     if (active) {
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
+        for (int u = 0; u < K::V; ++u)
             sbuf[b * SP + pad16(j + u * Q)] = v[0][u];
     }
     __syncthreads();
@@ -404,16 +417,16 @@ struct ColStage {
 // the fold of the odd half reuses them afterwards.
 constexpr int kColWalk = 4;
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_THREADS) k_col(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, P = 2 * N, QS = quarter_stride(N), HQ = quarter_half(N);
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -471,9 +484,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
             issue(1);
         cp_commit();
 
-        C acc[2][16];
+        C acc[2][K::V];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < K::V; ++u) {
             acc[0][u] = hmk<C>(T(0), T(0));
             acc[1][u] = hmk<C>(T(0), T(0));
         }
@@ -486,16 +499,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
             const ColInput ci = a.ins[w.in_begin + k / 3];
             const int rows = a.slabs[ci.slab].rows;
             const int f = k % 3;
-            C v[1][16];
+            C v[1][K::V];
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     C x = hmk<C>(T(0), T(0));
                     if (n < rows) {
                         x = col[n];
                         if (b)
-                            x = hmul(x, twist(tw, tl, j, u));
+                            x = hmul(x, twist_v<C, K::V>(tw, tl, N, j, u));
                     }
                     v[0][u] = x;
                 }
@@ -510,7 +523,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                     const T mx = (f == 2) ? T(-1) : T(1);
                     const T my = (f == 2) ? T(1) : T(-1);
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int kp = j + u * Q;
                         const bool hi = 2 * kp + b > N;
                         const int q = hi ? N - kp - b : kp;
@@ -528,7 +541,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                     // the potential alone: P0 real, Px Py imaginary; mirror signs + P0 Px, - Py
                     const T mx = (f == 2) ? T(-1) : T(1);
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int kp = j + u * Q;
                         const bool hi = 2 * kp + b > N;
                         const int q = hi ? N - kp - b : kp;
@@ -542,11 +555,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                     const C *sx = reinterpret_cast<const C *>(st + (size_t)N * sizeof(C)), *sy = sx + N;
                     if (ci.kind == SPEC_FULL_PHI) {
 #pragma unroll
-                        for (int u = 0; u < 16; ++u)
+                        for (int u = 0; u < K::V; ++u)
                             acc[0][u] = hadd(acc[0][u], hmul(sx[j + u * Q], v[0][u]));
                     } else {
 #pragma unroll
-                        for (int u = 0; u < 16; ++u) {
+                        for (int u = 0; u < K::V; ++u) {
                             acc[0][u] = hadd(acc[0][u], hmul(sx[j + u * Q], v[0][u]));
                             acc[1][u] = hadd(acc[1][u], hmul(sy[j + u * Q], v[0][u]));
                         }
@@ -554,7 +567,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                 } else if (ci.kind == SPEC_FULL_PHI) {
                     const C *sx = reinterpret_cast<const C *>(a.spec) + ci.spec_off + ((size_t)f * (N + 1) + kx) * P;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int ky = 2 * (j + u * Q) + b;
                         acc[0][u] = hadd(acc[0][u], hmul(__ldg(sx + ky), v[0][u]));
                     }
@@ -562,7 +575,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                     const C *sx = reinterpret_cast<const C *>(a.spec) + ci.spec_off + ((size_t)f * (N + 1) + kx) * P;
                     const C *sy = reinterpret_cast<const C *>(a.spec) + ci.spec_off + ((size_t)(3 + f) * (N + 1) + kx) * P;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int ky = 2 * (j + u * Q) + b;
                         acc[0][u] = hadd(acc[0][u], hmul(__ldg(sx + ky), v[0][u]));
                         acc[1][u] = hadd(acc[1][u], hmul(__ldg(sy + ky), v[0][u]));
@@ -581,7 +594,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                 for (int comp = 0; comp < 2; ++comp) {
                     C *dst = a.partial + ((((size_t)w.slot * 2 + b) * 2 + comp) * (N + 1) + kx) * N;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u)
+                    for (int u = 0; u < K::V; ++u)
                         dst[j + u * Q] = acc[comp][u];
                 }
             }
@@ -599,9 +612,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
         if (b == 1 && active) {
             C *dst = cluster.map_shared_rank(fold, 0);
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
-                const C w = twist(tw, tl, j, u);
+                const C w = twist_v<C, K::V>(tw, tl, N, j, u);
                 dst[n] = hmulc(acc[0][u], w);
                 if (two)
                     dst[N + n] = hmulc(acc[1][u], w);
@@ -611,7 +624,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
         if (b == 0 && active) {
             C *dst = a.bwd + o.off;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
                 if (n < o.rows) {
                     dst[bwd_index(N, o.rows, 0, kx, n)] = hadd(acc[0][u], fold[n]);
@@ -868,16 +881,16 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_w(SolveArg
 // memory.  Shared memory: twiddle area | sbuf[2 SPC] (the two exchange buffers,
 // then the 2N fold) | fld[3][N].
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_THREADS) k_col_g(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col_g(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, P = 2 * N;
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_G);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -900,18 +913,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
     cp_commit();
     cp_wait<0>();
     __syncthreads();
-    C v[1][16];
+    C v[1][K::V];
     for (int f = 0; f < 3; ++f) {
         if (active) {
             const C *col = a.fwd + sl.off + ((size_t)f * (N + 1) + kx) * sl.rows;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
                 C x = hmk<C>(T(0), T(0));
                 if (n < sl.rows) {
                     x = col[n];
                     if (b)
-                        x = hmul(x, twist(tw, tl, j, u));
+                        x = hmul(x, twist_v<C, K::V>(tw, tl, N, j, u));
                 }
                 v[0][u] = x;
             }
@@ -919,7 +932,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
         fft_ct<C, false, LOGN, 1, TC>(v, sbuf, SPC, j, active, tw, &tcx);
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
+            for (int u = 0; u < K::V; ++u)
                 fld[f * N + u * Q + j] = v[0][u];  // read back by this thread only
         }
     }
@@ -928,10 +941,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
     for (int q = 0; q < g.out_count; ++q) {
         const ColOutput o = a.outs[g.out_begin + q];
         const ColInput ci = a.ins[o.in_begin];
-        C acc[2][16];
+        C acc[2][K::V];
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 acc[0][u] = hmk<C>(T(0), T(0));
                 acc[1][u] = hmk<C>(T(0), T(0));
             }
@@ -940,7 +953,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                 for (int f = 0; f < 3; ++f) {
                     const C *sx = spec + ci.spec_off + ((size_t)f * (N + 1) + kx) * P;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int ky = 2 * (j + u * Q) + b;
                         acc[0][u] = hadd(acc[0][u], hmul(__ldg(sx + ky), fld[f * N + u * Q + j]));
                     }
@@ -951,7 +964,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
                     const C *sx = spec + ci.spec_off + ((size_t)f * (N + 1) + kx) * P;
                     const C *sy = spec + ci.spec_off + ((size_t)(3 + f) * (N + 1) + kx) * P;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int ky = 2 * (j + u * Q) + b;
                         const C x = fld[f * N + u * Q + j];
                         acc[0][u] = hadd(acc[0][u], hmul(__ldg(sx + ky), x));
@@ -966,8 +979,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
         if (b == 1 && active) {
             C *dst = cluster.map_shared_rank(sbuf, 0);
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const C w = twist(tw, tl, j, u);
+            for (int u = 0; u < K::V; ++u) {
+                const C w = twist_v<C, K::V>(tw, tl, N, j, u);
                 dst[j + u * Q] = hmulc(acc[0][u], w);
                 dst[N + j + u * Q] = hmulc(acc[1][u], w);
             }
@@ -976,7 +989,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
         if (b == 0 && active) {
             C *out = a.bwd + o.off;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
                 if (n < o.rows) {
                     out[bwd_index(N, o.rows, 0, kx, n)] = hadd(acc[0][u], sbuf[n]);
@@ -1119,16 +1132,16 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_gw(SolveAr
 // in k_col.  Shared memory: twiddle area | two exchange buffers (dual inverse),
 // reused for the fold.
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_THREADS) k_col_sum(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col_sum(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q;
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_SUM);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -1148,9 +1161,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
     const ColOutput o = a.outs[sm.out];
     cp_block(tw, a.tw, tw_bytes<C>(a.tw_entries));
     cp_commit();
-    C acc[2][16];
+    C acc[2][K::V];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < K::V; ++u) {
         acc[0][u] = hmk<C>(T(0), T(0));
         acc[1][u] = hmk<C>(T(0), T(0));
     }
@@ -1161,7 +1174,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
             for (int comp = 0; comp < 2; ++comp) {
                 const C *src = a.partial + ((((size_t)(sm.slot_begin + k) * 2 + b) * 2 + comp) * (N + 1) + kx) * N;
 #pragma unroll
-                for (int u = 0; u < 16; ++u)
+                for (int u = 0; u < K::V; ++u)
                     acc[comp][u] = hadd(acc[comp][u], src[j + u * Q]);
             }
         }
@@ -1174,9 +1187,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
     if (b == 1 && active) {
         C *dst = cluster.map_shared_rank(fold, 0);
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < K::V; ++u) {
             const int n = j + u * Q;
-            const C tw_n = twist(tw, tl, j, u);
+            const C tw_n = twist_v<C, K::V>(tw, tl, N, j, u);
             dst[n] = hmulc(acc[0][u], tw_n);
             dst[N + n] = hmulc(acc[1][u], tw_n);
         }
@@ -1185,7 +1198,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
     if (b == 0 && active) {
         C *dst = a.bwd + o.off;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < K::V; ++u) {
             const int n = j + u * Q;
             if (n < o.rows) {
                 dst[bwd_index(N, o.rows, 0, kx, n)] = hadd(acc[0][u], fold[n]);
@@ -1204,15 +1217,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN>::COL_TH
 // one output, 8 bytes otherwise -- and the next gather is issued as soon as
 // the current one has been read into registers, so it overlaps the transform.
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_inv(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS) k_row_inv(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, SP = K::SP_ROW, P = 2 * N;
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::ROW_THREADS, 1);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::ROW_THREADS, 1);
     constexpr int TCR = tc_round(LOGN, TCT, KK_ROW_INV);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -1270,10 +1283,10 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_inv(SolveArgs
         const int nout = N / rc.m;
         cp_wait<0>();
         __syncthreads();
-        C v[1][16];
+        C v[1][K::V];
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int kx = 2 * (j + u * Q) + b;
                 const int k2 = kx <= N ? kx : P - kx;
                 const C A = stg[2 * k2], B = stg[2 * k2 + 1];
@@ -1291,16 +1304,16 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_inv(SolveArgs
         __syncthreads();
         if (active && b == 1) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
-                sbuf[pad16(n)] = hmulc(v[0][u], twist(tw, twl, j, u));
+                sbuf[pad16(n)] = hmulc(v[0][u], twist_v<C, K::V>(tw, twl, N, j, u));
             }
         }
         __syncthreads();
         if (active && b == 0) {
             T *Oc = O + comp * 2 * N;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
                 if (n < nout) {
                     const C y = hadd(v[0][u], sbuf[pad16(n)]);
@@ -1340,16 +1353,16 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_inv(SolveArgs
 // The tensor-core instances are launched with fewer CTAs in x (the resident
 // CTAs shared among the patches), each walking those items in turn.
 template <typename T, int LOGN, bool BATCH, bool TC, int NC>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !TC && NC == 1 ? 2 : 1)
+__global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS, sizeof(T) == 4 && !TC && NC == 1 ? 2 : 1)
     k_row_inv1(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, SP = K::SP_ROW, P = 2 * N;
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::ROW_THREADS, NC);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::ROW_THREADS, NC);
     constexpr int TCR = tc_round(LOGN, TCT, NC == 1 ? KK_ROW_INV1 : KK_ROW_INV2);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -1391,12 +1404,12 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
         cp_commit();
         cp_wait<0>();
         __syncthreads();
-        C v[NC][16];
+        C v[NC][K::V];
         if (active) {
 #pragma unroll
             for (int c = 0; c < NC; ++c)
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int kx = 2 * (j + u * Q) + b;
                     const int k2 = kx <= N ? kx : P - kx;  // same parity as kx
                     const C *pr = stg + 2 * ((c * 2 + b) * HALF + (k2 >> 1));
@@ -1421,9 +1434,9 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
         __syncthreads();
         if (active && b == 1) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
-                const C w = twist(tw, twl, j, u);
+                const C w = twist_v<C, K::V>(tw, twl, N, j, u);
 #pragma unroll
                 for (int c = 0; c < NC; ++c)
                     sbuf[c * SP + pad16(n)] = hmulc(v[c][u], w);
@@ -1435,7 +1448,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, sizeof(T) == 4 && !
             for (int c = 0; c < NC; ++c) {
                 T *out = comp0 + c ? a.fy[tl] : a.fx[tl];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     const C y = hadd(v[c][u], sbuf[c * SP + pad16(n)]);
                     out[(size_t)j0 * N + n] = covered(a, tl, j0, n) ? T(0) : y.x;
@@ -1832,16 +1845,16 @@ __global__ void __launch_bounds__(KR2x<LOGN>::THREADS, 1) k_row_inv2x(const __gr
 // the others, and batches, take one row pair per CTA, which measured faster.
 // Shared memory: twiddle area | sigma rows[2][N] | sbuf[2 SP_ROW].
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_fwd_m(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS) k_row_fwd_m(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, 0);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
     using C2 = typename Cx<T>::C2;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, SP = K::SP_ROW;
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::ROW_THREADS, 1);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::ROW_THREADS, 1);
     constexpr int TCR = tc_round(LOGN, TCT, KK_ROW_FWD_M);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -1879,14 +1892,14 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_fwd_m(SolveAr
             if (bad)
                 rim_bad = 1;
         }
-        C v[1][16];
+        C v[1][K::V];
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int c = j + u * Q;
                 C z = hmk<C>(srow[c], srow[N + c]);
                 if (b)
-                    z = hmul(z, twist(tw, tl, j, u));
+                    z = hmul(z, twist_v<C, K::V>(tw, tl, N, j, u));
                 v[0][u] = z;
             }
         }
@@ -1900,7 +1913,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS) k_row_fwd_m(SolveAr
         __syncthreads();
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
+            for (int u = 0; u < K::V; ++u)
                 sbuf[b * SP + pad16(j + u * Q)] = v[0][u];
         }
         __syncthreads();
@@ -2274,16 +2287,16 @@ __global__ void __launch_bounds__(KF3x<LOGN>::THREADS, 1) k_row_fwd3x(const __gr
 // (exchanges, then the fold) | park[N] (Fy^ in slot order).
 template <typename T, int LOGN, bool BATCH, bool TC>
 __global__ void __cluster_dims__(2, 1, 1)
-    __launch_bounds__(KShape<LOGN>::COL_THREADS, sizeof(T) == 4 && !TC ? 3 : 1) k_col_m(SolveArgs<T> a0, BatchView<T> bv)
+    __launch_bounds__(KShape<LOGN, TC>::COL_THREADS, sizeof(T) == 4 && !TC ? 3 : 1) k_col_m(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, 0);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, QS = quarter_stride(N), HQ = quarter_half(N);
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::COL_THREADS, 1);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 1);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_M);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -2306,24 +2319,24 @@ __global__ void __cluster_dims__(2, 1, 1)
     for (int kx = blockIdx.x >> 1; kx <= N; kx += WALK ? (int)(gridDim.x >> 1) : N + 1) {
         const T *gxr = reinterpret_cast<const T *>(a.spec) + (size_t)kx * QS + b * HQ;
         const T *gyr = reinterpret_cast<const T *>(a.spec) + ((size_t)(N + 1) + kx) * QS + b * HQ;
-        C v[1][16];
+        C v[1][K::V];
         if (active) {
             const C *col = a.fwd + (size_t)kx * N;
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
+            for (int u = 0; u < K::V; ++u)
                 v[0][u] = col[j + u * Q];
         }
         cp_wait<0>();
         __syncthreads();
         if (active && b) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u)
-                v[0][u] = hmul(v[0][u], twist(tw, tl, j, u));
+            for (int u = 0; u < K::V; ++u)
+                v[0][u] = hmul(v[0][u], twist_v<C, K::V>(tw, tl, N, j, u));
         }
         fft_ct<C, false, LOGN, 1, TC>(v, sbuf, SPC, j, active, tw, &tcx);
         if (active) {
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int kp = j + u * Q;
                 const bool hi = 2 * kp + b > N;
                 const int q = hi ? N - kp - b : kp;
@@ -2338,7 +2351,7 @@ __global__ void __cluster_dims__(2, 1, 1)
         for (int comp = 0; comp < 2; ++comp) {
             if (comp == 1 && active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u)
+                for (int u = 0; u < K::V; ++u)
                     v[0][u] = park[u * Q + j];
             }
             // y[n] = even[n] + W_P^{-n} odd[n]
@@ -2347,13 +2360,13 @@ __global__ void __cluster_dims__(2, 1, 1)
             if (b == 1 && active) {
                 C *dst = cluster.map_shared_rank(sbuf, 0);
 #pragma unroll
-                for (int u = 0; u < 16; ++u)
-                    dst[j + u * Q] = hmulc(v[0][u], twist(tw, tl, j, u));
+                for (int u = 0; u < K::V; ++u)
+                    dst[j + u * Q] = hmulc(v[0][u], twist_v<C, K::V>(tw, tl, N, j, u));
             }
             cluster.sync();
             if (b == 0 && active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     out[bwd_index(N, N, comp, kx, n)] = hadd(v[0][u], sbuf[n]);
                 }
@@ -2373,16 +2386,16 @@ __global__ void __cluster_dims__(2, 1, 1)
 // sequence and the 2N fold reuse sbuf + column.
 template <typename T, int LOGN, bool BATCH, bool TC>
 __global__ void __cluster_dims__(2, 1, 1)
-    __launch_bounds__(KShape<LOGN>::COL_THREADS, sizeof(T) == 4 && !TC ? 2 : 1) k_col_md(SolveArgs<T> a0, BatchView<T> bv)
+    __launch_bounds__(KShape<LOGN, TC>::COL_THREADS, sizeof(T) == 4 && !TC ? 2 : 1) k_col_md(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, 0);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, QS = quarter_stride(N), HQ = quarter_half(N);
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_MD);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -2412,22 +2425,22 @@ __global__ void __cluster_dims__(2, 1, 1)
         cp_commit();
         cp_wait<0>();
         __syncthreads();
-        C acc[2][16];
+        C acc[2][K::V];
         {
-            C v[1][16];
+            C v[1][K::V];
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     C x = col[j + u * Q];
                     if (b)
-                        x = hmul(x, twist(tw, tl, j, u));
+                        x = hmul(x, twist_v<C, K::V>(tw, tl, N, j, u));
                     v[0][u] = x;
                 }
             }
             fft_ct<C, false, LOGN, 1, TC>(v, sbuf, SPC, j, active, tw, &tcx);
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int kp = j + u * Q;
                     const bool hi = 2 * kp + b > N;
                     const int q = hi ? N - kp - b : kp;
@@ -2444,9 +2457,9 @@ __global__ void __cluster_dims__(2, 1, 1)
         if (b == 1 && active) {
             C *dst = cluster.map_shared_rank(fold, 0);
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
-                const C w = twist(tw, tl, j, u);
+                const C w = twist_v<C, K::V>(tw, tl, N, j, u);
                 dst[n] = hmulc(acc[0][u], w);
                 dst[N + n] = hmulc(acc[1][u], w);
             }
@@ -2455,7 +2468,7 @@ __global__ void __cluster_dims__(2, 1, 1)
         if (b == 0 && active) {
             C *dst = a.bwd;
 #pragma unroll
-            for (int u = 0; u < 16; ++u) {
+            for (int u = 0; u < K::V; ++u) {
                 const int n = j + u * Q;
                 dst[bwd_index(N, N, 0, kx, n)] = hadd(acc[0][u], fold[n]);
                 dst[bwd_index(N, N, 1, kx, n)] = hadd(acc[1][u], fold[N + n]);
@@ -2480,16 +2493,16 @@ __global__ void __cluster_dims__(2, 1, 1)
 // exchange buffers, half b's two sequences at sbuf + 2 b SPC (then the fold).
 // NC = 2: the forces (Gx, Gy); NC = 1: the potential (Gphi alone, one inverse transform).
 template <typename T, int LOGN, bool BATCH, bool TC, int NC = 2>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS, 1) k_col_mw(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, 0);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
     using C = typename Cx<T>::C;
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     constexpr int N = K::N, Q = K::Q, QS = quarter_stride(N), HQ = quarter_half(N);
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN>::ROW_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::ROW_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_MW);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -2521,15 +2534,15 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
     for (int kx = blockIdx.x; kx <= N; kx += gridDim.x) {
         cp_wait<0>();
         __syncthreads();  // column kx staged; the previous column's fold has been read
-        C acc[2][16];
+        C acc[2][K::V];
         {
-            C v[1][16];
+            C v[1][K::V];
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     C x = col[j + u * Q];
                     if (b)
-                        x = hmul(x, twist(tw, tl, j, u));
+                        x = hmul(x, twist_v<C, K::V>(tw, tl, N, j, u));
                     v[0][u] = x;
                 }
             }
@@ -2539,7 +2552,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
                 if (active) {
                     const T *gx_r = gsp + (2 * b) * HQ, *gy_r = gsp + (2 * b + 1) * HQ;
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
+                    for (int u = 0; u < K::V; ++u) {
                         const int kp = j + u * Q;
                         const bool hi = 2 * kp + b > N;
                         const int q = hi ? N - kp - b : kp;
@@ -2552,7 +2565,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
             } else if (active) {
                 const T *gp_r = gsp + (2 * b) * HQ;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int kp = j + u * Q;
                     const int q = 2 * kp + b > N ? N - kp - b : kp;
                     const T gp = gp_r[q];  // Gphi real, even in ky
@@ -2571,10 +2584,10 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
             C *fold = sbuf;
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     if (b == 1 && u < 8)
-                        fold[n] = hmulc(acc[0][u], twist(tw, tl, j, u));
+                        fold[n] = hmulc(acc[0][u], twist_v<C, K::V>(tw, tl, N, j, u));
                     else if (b == 0 && u >= 8)
                         fold[n] = acc[0][u];
                 }
@@ -2582,12 +2595,12 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
             __syncthreads();
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     if (b == 0 && u < 8)
                         dst[bwd_index(N, N, 0, kx, n)] = hadd(acc[0][u], fold[n]);
                     else if (b == 1 && u >= 8)
-                        dst[bwd_index(N, N, 0, kx, n)] = hadd(fold[n], hmulc(acc[0][u], twist(tw, tl, j, u)));
+                        dst[bwd_index(N, N, 0, kx, n)] = hadd(fold[n], hmulc(acc[0][u], twist_v<C, K::V>(tw, tl, N, j, u)));
                 }
             }
         } else {
@@ -2598,10 +2611,10 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
             C *fold = sbuf;
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     if (b == 1)
-                        fold[n] = hmulc(acc[0][u], twist(tw, tl, j, u));
+                        fold[n] = hmulc(acc[0][u], twist_v<C, K::V>(tw, tl, N, j, u));
                     else
                         fold[N + n] = acc[1][u];
                 }
@@ -2609,12 +2622,12 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_mw(SolveAr
             __syncthreads();
             if (active) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
+                for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
                     if (b == 0)
                         dst[bwd_index(N, N, 0, kx, n)] = hadd(acc[0][u], fold[n]);
                     else
-                        dst[bwd_index(N, N, 1, kx, n)] = hadd(fold[N + n], hmulc(acc[1][u], twist(tw, tl, j, u)));
+                        dst[bwd_index(N, N, 1, kx, n)] = hadd(fold[N + n], hmulc(acc[1][u], twist_v<C, K::V>(tw, tl, N, j, u)));
                 }
             }
         }
@@ -2779,13 +2792,13 @@ struct KSmem {
     {
         return TC ? tc_smem_bytes(tc_round(LOGN, tc_tiles(threads, B), kind)) : 0;
     }
-    static size_t rtc(int kind) { return tc(KShape<LOGN>::ROW_THREADS, 1, kind); }
-    static size_t ctc(int kind) { return tc(KShape<LOGN>::COL_THREADS, 2, kind); }
+    static size_t rtc(int kind) { return tc(KShape<LOGN, TC>::ROW_THREADS, 1, kind); }
+    static size_t ctc(int kind) { return tc(KShape<LOGN, TC>::COL_THREADS, 2, kind); }
     static size_t tw() { return tw_bytes<C>(tw_layout(F16<LOGN>::twlen, N).entries); }
     static size_t row_fwd()
     {
         // the staged rows (at most 4 N reals) fit in the exchange buffers' 2 SP_ROW complex
-        return rtc(KK_ROW_FWD) + tw() + 2 * (size_t)KShape<LOGN>::SP_ROW * sizeof(C);
+        return rtc(KK_ROW_FWD) + tw() + 2 * (size_t)KShape<LOGN, TC>::SP_ROW * sizeof(C);
     }
     static size_t col()
     {
@@ -2795,23 +2808,23 @@ struct KSmem {
     static size_t row_inv()
     {
         return rtc(KK_ROW_INV) + tw() + ((2 * (size_t)(N + 1) * sizeof(C) + 15) & ~(size_t)15) +
-               2 * (size_t)KShape<LOGN>::SP_ROW * sizeof(C) + 4 * (size_t)N * sizeof(T);
+               2 * (size_t)KShape<LOGN, TC>::SP_ROW * sizeof(C) + 4 * (size_t)N * sizeof(T);
     }
     static size_t row_inv1(int nc)
     {
         const size_t stage = (size_t)nc * 2 * (N / 2 + 1) * 2 * sizeof(C);  // [comp][parity][N/2 + 1] pairs
-        const size_t xbuf = (size_t)nc * 2 * KShape<LOGN>::SP_ROW * sizeof(C);
-        return tc(KShape<LOGN>::ROW_THREADS, nc, nc == 1 ? KK_ROW_INV1 : KK_ROW_INV2) + tw() +
+        const size_t xbuf = (size_t)nc * 2 * KShape<LOGN, TC>::SP_ROW * sizeof(C);
+        return tc(KShape<LOGN, TC>::ROW_THREADS, nc, nc == 1 ? KK_ROW_INV1 : KK_ROW_INV2) + tw() +
                (stage > xbuf ? stage : xbuf);
     }
     static size_t row_inv1t() { return row_inv1t_body<T, LOGN>() + tw() + 16 + 128; }  // + mbarrier, alignment slack
     static size_t row_fwd_m()
     {
-        return rtc(KK_ROW_FWD_M) + tw() + 2 * (size_t)N * sizeof(T) + 2 * (size_t)KShape<LOGN>::SP_ROW * sizeof(C);
+        return rtc(KK_ROW_FWD_M) + tw() + 2 * (size_t)N * sizeof(T) + 2 * (size_t)KShape<LOGN, TC>::SP_ROW * sizeof(C);
     }
     static size_t col_m()
     {
-        return tc(KShape<LOGN>::COL_THREADS, 1, KK_COL_M) + tw() + (size_t)col_sp<C>(N) * sizeof(C) +
+        return tc(KShape<LOGN, TC>::COL_THREADS, 1, KK_COL_M) + tw() + (size_t)col_sp<C>(N) * sizeof(C) +
                (size_t)N * sizeof(C);
     }
     static size_t col_gw()
@@ -2820,7 +2833,7 @@ struct KSmem {
     }
     static size_t col_g()
     {
-        return tc(KShape<LOGN>::COL_THREADS, 2, KK_COL_G) + tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) +
+        return tc(KShape<LOGN, TC>::COL_THREADS, 2, KK_COL_G) + tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) +
                3 * (size_t)N * sizeof(C);
     }
     static size_t col_sum()
@@ -2830,7 +2843,7 @@ struct KSmem {
     }
     static size_t col_mw()
     {
-        return tc(KShape<LOGN>::ROW_THREADS, 2, KK_COL_MW) + tw() + (size_t)N * sizeof(C) +
+        return tc(KShape<LOGN, TC>::ROW_THREADS, 2, KK_COL_MW) + tw() + (size_t)N * sizeof(C) +
                4 * (size_t)quarter_half(N) * sizeof(T) + 4 * (size_t)col_sp<C>(N) * sizeof(C);
     }
     static size_t col_md()
@@ -2902,7 +2915,7 @@ inline int min_grid(int items, int resident, int count)
 template <typename T, int LOGN, bool TC>
 cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t st, const BatchView<T> *bv)
 {
-    using K = KShape<LOGN>;
+    using K = KShape<LOGN, TC>;
     using S = KSmem<T, LOGN, TC>;
     static std::atomic<unsigned long long> d[40];
     static std::atomic<int> res_mx[64], res_mx1[64];  // resident CTAs of the register-twiddle column pass (plans 0, 1)

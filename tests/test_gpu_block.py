@@ -51,14 +51,14 @@ def _worst(geom, got, ref, samp):
 
 
 NESTS = {
-    "256x2_corner": (W.Nest(n=256, levels=2, off=[(0, 0), (0, 128)]), ("fp32", "bf16x")),
+    "512x2_corner": (W.Nest(n=512, levels=2, off=[(0, 0), (0, 256)]), ("fp32", "bf16x")),
     "256x3_odd": (W.Nest(n=256, levels=3, off=[(0, 0), (37, 90), (101, 3)]), ("fp32", "bf16x")),
     "256x5": (W.Nest(n=256, levels=5, off=[(0, 0), (64, 65), (63, 7), (128, 64), (31, 33)]), ("fp32",)),
     "300x3_embedded": (W.Nest(n=300, levels=3, off=[(0, 0), (75, 11), (150, 80)]), ("fp32",)),
     "1024x4": (W.Nest(n=1024, levels=4, off=[(0, 0), (255, 256), (301, 4), (256, 511)]), ("fp32",)),
     "2048x2": (W.Nest(n=2048, levels=2, off=[(0, 0), (513, 700)]), ("fp32",)),
     "4096x2": (W.Nest(n=4096, levels=2, off=[(0, 0), (1025, 1000)]), ("fp32",)),
-    "two_patches256": (W.two_patch_forest(256), ("fp32",)),
+    "two_patches512": (W.two_patch_forest(512), ("fp32",)),
     "example4_256": (W.example4_forest(256), ("fp32",)),
 }
 
@@ -75,7 +75,7 @@ def test_block_pairs_against_oracle(lib, name, prec):
     assert _worst(geom, (gx, gy), (ox, oy), samp) <= tol(prec, geom.n)
 
 
-@pytest.mark.parametrize("name", ["256x2_corner", "256x3_odd", "256x5", "300x3_embedded"])
+@pytest.mark.parametrize("name", ["512x2_corner", "256x3_odd", "256x5", "300x3_embedded"])
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_block_pairs_equal_whole_grid_pairs(lib, name, prec):
     """A plan over its spectra budget runs the whole-grid passes on the same FP64 tables: the

@@ -188,6 +188,7 @@ struct sgf_plan {
     std::vector<RowContrib> contribs;
     std::vector<ColWork> work_all, work_main;  // k_col work lists: every output / the main outputs
     std::vector<ColGroup> groups;              // Case-3 output groups (k_col_g)
+    bool quarter_only = false;                 // every column input has quarter spectra, N >= 1024 (k_col_w's QO form)
     std::vector<ColSum> sums;                  // chunked outputs (k_col_sum)
     size_t partial_elems = 0;                  // complex elements of the chunk accumulators
     int contrib_begin[kMaxPatches + 1] = {};
@@ -281,6 +282,7 @@ struct sgf_batch {
         size_t map_fwd = 0, map_col = 0, map_inv1 = 0, map_inv = 0;  // int2 offsets in the map buffer
         int n_grp = 0, n_sum = 0;
         size_t map_grp = 0, map_sum = 0;  // Case-3 groups (k_col_g), chunked outputs (k_col_sum)
+        bool quarter_only = true;  // every column input of its plans has quarter spectra
         bool own = true;  // no finer patch has Case-3 outputs: k_row_inv1 for those too
     };
     std::vector<Group> groups;
@@ -992,6 +994,7 @@ void build_lists(sgf_plan *p)
     if (p->blk)
         build_blocks(p, off);
     p->in_set.clear();
+    p->quarter_only = N >= 1024 && std::all_of(p->ins.begin(), p->ins.end(), [](const ColInput &ci) { return spec_quarter(ci.kind); });
     for (auto &ci : p->ins) {
         p->in_set.push_back((int)ci.spec_off);
         ci.spec_off = p->sets[ci.spec_off].spec_off;
@@ -1648,6 +1651,12 @@ inline int general_fwd_pass(const sgf_plan *p)
     return p->sched.row_fwd == 2 ? PASS_ROW_FWD3X : p->sched.row_fwd == 1 ? PASS_ROW_FWD2 : PASS_ROW_FWD;
 }
 
+// General column pass of a schedule: a cluster per column, or both halves in one CTA.
+inline int general_col_pass(const sgf_schedule &s, bool quarter_only)
+{
+    return s.col_pass != 2 ? PASS_COL : quarter_only ? PASS_COL_WQ : PASS_COL_W;
+}
+
 // Zero-rim column pass of the plan's schedule.
 inline int col_m_pass(const sgf_plan *p)
 {
@@ -1700,7 +1709,7 @@ cudaError_t launch_col(const sgf_plan *p, const SolveArgs<T> &a, cudaStream_t st
         return launch_pass_n<T>(col_m_pass(p), p->logN, a, 1, st, nullptr, p->tc);
     }
     cudaError_t e;
-    const int colp = p->sched.col_pass == 2 ? PASS_COL_W : PASS_COL;  // both halves in one CTA, or a cluster
+    const int colp = general_col_pass(p->sched, p->quarter_only);
     if (p->sched.col_case3 == 1) {
         e = launch_pass_n<T>(colp, p->logN, a, (int)p->work_all.size(), st, nullptr, p->tc);
     } else {
@@ -2097,7 +2106,7 @@ sgf_status batch_launches(sgf_batch *bt, cudaStream_t st)
         dummy.N = 1 << g.logN;
         if ((e = launch_pass_n<T>(g.merged ? PASS_ROW_FWD_M : PASS_ROW_FWD, g.logN, dummy, g.n_fwd, gs, &vf, g.tc)) != cudaSuccess)
             return cuda_fail(e, "batched row_fwd launch");
-        const int colp = !g.merged              ? (g.sched.col_pass == 2 ? PASS_COL_W : PASS_COL)
+        const int colp = !g.merged              ? general_col_pass(g.sched, g.quarter_only)
                          : g.sched.col_pass == 1 ? PASS_COL_MD
                          : g.sched.col_pass >= 2 ? PASS_COL_MW  // k_col_mx has no batch form
                                                  : PASS_COL_M;
@@ -2266,6 +2275,7 @@ sgf_status batch_build(sgf_batch *bt)
             bt->groups.push_back(g);
             members.emplace_back();
         }
+        bt->groups[gidx[key]].quarter_only &= p->quarter_only;
         bt->groups[gidx[key]].own &= own;
         members[gidx[key]].push_back(k);
         bt->plan_group.push_back(gidx[key]);

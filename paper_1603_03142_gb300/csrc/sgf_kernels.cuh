@@ -644,12 +644,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
 // input of Cases 2 and 3 (x and y tables, 2N bins each), so that those are
 // copied in ahead like the column instead of being loaded in the product (two
 // CTAs per SM still fit at N = 1024, one at 2048, where it measured faster all
-// the same; at 4096 two stages would not fit).
-template <typename T, int LOGN>
+// the same; at 4096 two stages would not fit).  QO: plans whose inputs all have
+// quarter spectra (a uniform grid, block convolutions for the other pairs) stage
+// no full rows.
+template <typename T, int LOGN, bool QO>
 struct ColWStage {
     using C = typename Cx<T>::C;
     static constexpr int N = 1 << LOGN;
-    static constexpr bool FULL = LOGN <= 11;
+    static constexpr bool FULL = LOGN <= 11 && !QO;
     static constexpr size_t QB = 4 * (size_t)quarter_half(N) * sizeof(T);
     static constexpr size_t FB = FULL ? 2 * (size_t)(2 * N) * sizeof(C) : 0;
     static constexpr size_t BYTES = (size_t)N * sizeof(C) + (QB > FB ? QB : FB);
@@ -672,8 +674,17 @@ struct ColWStage {
 // ColWStage) the full rows [x, y][2N] complex }.  The dual
 // inverse transforms of half b use 2 SPC from sbuf + 2 b SPC (reaching over the
 // stages, free by then), and the fold reuses the start.
-template <typename T, int LOGN, bool BATCH>
-__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_w(SolveArgs<T> a0, BatchView<T> bv)
+//
+// QO: 16 warps per SM (128 registers a thread; the smaller stage fits four CTAs at
+// N = 1024, two at 2048) in place of 8 with up to 225 registers: three fields and two
+// components per column are a long chain between barriers, and more columns in
+// flight hide it better than a few spilled registers cost.  Column pass before ->
+// after: 2048^2 2 levels 351 -> 268 us, 1024^2 3 levels 134 -> 109; 1024^2 uniform
+// solve 94 -> 81, 2048^2 315 -> 273.  N >= 1024: the columns of a 512^2 grid fit the
+// SMs at once, and its solve gained nothing (35.6 -> 36.9).
+template <typename T, int LOGN, bool BATCH, bool QO = false>
+__global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, QO ? 512 / KShape<LOGN>::ROW_THREADS : 1)
+    k_col_w(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.x] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
@@ -687,7 +698,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_w(SolveArg
     C *tw = reinterpret_cast<C *>(smem_raw);
     C *sbuf = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));
     unsigned char *stage_base = reinterpret_cast<unsigned char *>(sbuf + 2 * SPC);
-    using CS = ColWStage<T, LOGN>;
+    using CS = ColWStage<T, LOGN, QO>;
     constexpr size_t stage_bytes = CS::BYTES;
     const int kx = BATCH ? (int)blockIdx.y : (int)blockIdx.x;
     const ColWork w = a.col_list[wm.y];
@@ -2804,7 +2815,8 @@ struct KSmem {
     {
         return ctc(KK_COL) + tw() + (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColStage<T, LOGN, TC>::BYTES;
     }
-    static size_t col_w() { return tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColWStage<T, LOGN>::BYTES; }
+    static size_t col_w() { return tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColWStage<T, LOGN, false>::BYTES; }
+    static size_t col_wq() { return tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColWStage<T, LOGN, true>::BYTES; }
     static size_t row_inv()
     {
         return rtc(KK_ROW_INV) + tw() + ((2 * (size_t)(N + 1) * sizeof(C) + 15) & ~(size_t)15) +
@@ -2917,7 +2929,7 @@ cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t
 {
     using K = KShape<LOGN, TC>;
     using S = KSmem<T, LOGN, TC>;
-    static std::atomic<unsigned long long> d[40];
+    static std::atomic<unsigned long long> d[48];
     static std::atomic<int> res_mx[64], res_mx1[64];  // resident CTAs of the register-twiddle column pass (plans 0, 1)
     static std::atomic<int> res_rx[64], res_rx1[64];  // and of the register-twiddle inverse row pass
     static std::atomic<int> res_r2[64], res_r21[64];  // and of its two-pair form
@@ -2997,6 +3009,9 @@ cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t
             if ((S::col_w() <= kMaxDynSmem &&
                  ((e = ensure_smem(k_col_w<T, LOGN, false>, S::col_w(), d[23])) != cudaSuccess ||
                   (e = ensure_smem(k_col_w<T, LOGN, true>, S::col_w(), d[24])) != cudaSuccess)) ||
+                (LOGN >= 10 && S::col_wq() <= kMaxDynSmem &&
+                 ((e = ensure_smem(k_col_w<T, LOGN, false, true>, S::col_wq(), d[40])) != cudaSuccess ||
+                  (e = ensure_smem(k_col_w<T, LOGN, true, true>, S::col_wq(), d[41])) != cudaSuccess)) ||
                 (S::col_gw() <= kMaxDynSmem &&
                  ((e = ensure_smem(k_col_gw<T, LOGN, false>, S::col_gw(), d[26])) != cudaSuccess ||
                   (e = ensure_smem(k_col_gw<T, LOGN, true>, S::col_gw(), d[27])) != cudaSuccess)) ||
@@ -3153,6 +3168,17 @@ cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t
             if (S::col_w() > kMaxDynSmem)
                 return cudaErrorInvalidConfiguration;
             SGF_LAUNCH((k_col_w<T, LOGN, false>), (k_col_w<T, LOGN, true>), 23, S::col_w(),
+                       batch ? dim3(count, K::N + 1) : dim3(K::N + 1, count), K::ROW_THREADS)
+        } else {
+            return cudaErrorInvalidValue;
+        }
+        break;
+    }
+    case PASS_COL_WQ: {
+        if constexpr (!TC && LOGN >= 10 && sizeof(T) == 4) {
+            if (S::col_wq() > kMaxDynSmem)
+                return cudaErrorInvalidConfiguration;
+            SGF_LAUNCH((k_col_w<T, LOGN, false, true>), (k_col_w<T, LOGN, true, true>), 40, S::col_wq(),
                        batch ? dim3(count, K::N + 1) : dim3(K::N + 1, count), K::ROW_THREADS)
         } else {
             return cudaErrorInvalidValue;

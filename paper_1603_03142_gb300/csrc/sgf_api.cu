@@ -572,14 +572,14 @@ size_t blk_set_elems(const sgf_plan *p, const GenSet &g)
 // anyway, and so they do for FP32 potentials of a few patches on two levels at 256
 // (us per solve, whole-grid / block: 65.5 / 73.8; forces 76.8 / 79.1, but blocks save
 // a batch more; eight patches 556 / 327; three levels 258 / 147; FP64 forces 528 / 434).
-// SGF_BF16X plans of four levels and more stay with the whole-grid passes: the
+// SGF_BF16X plans of three levels and more stay with the whole-grid passes: the
 // block transforms run in FP32, and from that depth on the split-BF16 rounding
-// they leave out moves the finest level's forces by more than 2e-5 (2-norm;
-// 2.7e-5 at 4 levels, 1.5e-5 at 3, 0.7e-5 at 2).
+// they leave out moves the finest level's forces by up to 2.3e-5 (2-norm over 83
+// nests; 2.7e-5 at four levels), where 2 levels stay below 0.7e-5.
 bool blk_applies(const sgf_plan *p)
 {
     return !p->merged && p->fo.depth > 1 && p->N >= 256 && (p->N >> (p->fo.depth - 1)) >= 16 &&
-           (p->N > 256 || p->fo.depth > 2 || p->fo.K > 3 || !p->pot || p->esize == 8) && !(p->tc && p->fo.depth > 3);
+           (p->N > 256 || p->fo.depth > 2 || p->fo.K > 3 || !p->pot || p->esize == 8) && !(p->tc && p->fo.depth > 2);
 }
 
 // Twiddle area of the B-point block transforms within Spectra::twb (complex entries).

@@ -341,12 +341,17 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
         return fail(SGF_EINVAL, "NULL argument");
     Pending p;
     p.r = *r;
-    // FP32 and SGF_BF16X requests of a shape share its spectra: from four levels on, where
-    // SGF_BF16X plans keep the whole-grid passes, every request of the shape does
-    p.whole_grid = r->desc.levels >= 4;
-    sgf_status rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, p.whole_grid, &p.ws, &p.spectra, &p.build);
+    // FP32 and SGF_BF16X requests of a shape share its spectra: from three levels on, where
+    // SGF_BF16X plans keep the whole-grid passes, every request of the shape does (the
+    // per-shape cap goes by sgf_plan_estimate all the same)
+    p.whole_grid = r->desc.levels >= 3;
+    size_t pub_ws = 0, pub_spectra = 0, pub_build = 0;
+    sgf_status rc = sgf_plan_estimate(&r->desc, r->precision, r->plan_flags, &pub_ws, &pub_spectra, &pub_build);
+    if (rc == SGF_OK)
+        rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, p.whole_grid, &p.ws, &p.spectra, &p.build);
     if (rc != SGF_OK)
         return rc;
+    const size_t shape_bytes = std::max(p.spectra + p.build, pub_spectra + pub_build);
     if (r->plan_flags & SGF_PLAN_POTENTIAL)
         return fail(SGF_EUNSUPPORTED, "request %llu: the request loop solves forces, not SGF_PLAN_POTENTIAL",
                     (unsigned long long)r->id);
@@ -366,7 +371,7 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
         if (rc != SGF_OK)
             return rc;
     }
-    if (sv->cfg.max_shape_bytes && p.spectra + p.build > sv->cfg.max_shape_bytes &&
+    if (sv->cfg.max_shape_bytes && shape_bytes > sv->cfg.max_shape_bytes &&
         (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0 && p.build < sv->cfg.max_shape_bytes) {
         // served by plans over a spectra budget: resident sets and a window within the budget,
         // the generator's workspace kept by every slot's plan
@@ -380,10 +385,10 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
         }
     }
     const size_t worst = p.ws + p.io + p.spectra + p.build;
-    if (sv->cfg.max_shape_bytes && p.spectra + p.build > sv->cfg.max_shape_bytes) {
+    if (sv->cfg.max_shape_bytes && !p.stream_budget && shape_bytes > sv->cfg.max_shape_bytes) {
         sv->st.rejected++;
         return fail(SGF_ENOMEM, "request %llu: its shape needs %zu bytes of spectra and generator memory, above "
-                    "max_shape_bytes %zu", (unsigned long long)r->id, p.spectra + p.build, sv->cfg.max_shape_bytes);
+                    "max_shape_bytes %zu", (unsigned long long)r->id, shape_bytes, sv->cfg.max_shape_bytes);
     }
     if (worst > sv->cfg.hbm_budget) {
         sv->st.rejected++;

@@ -142,7 +142,8 @@ struct BlkTarget {
     };
     std::vector<Term> terms;
     size_t a_off = 0;
-    int m2 = 0, F = 0;
+    int m2 = 0, F = 0, logm = 0, logB = 0;
+    int sym = kMirrorX | kMirrorY;  // mirror symmetry that all terms have
 };
 
 struct SetKey {
@@ -209,7 +210,7 @@ struct sgf_plan {
     std::vector<MacItem> mitems;
     std::vector<MacTerm> mterms;
     std::vector<size_t> mxo, mao;
-    int mac_blocks = 0;
+    MacLaunch mac;
     size_t blk_x_elems = 0, blk_elems = 0;  // complex elements: source fields; source and target fields
     const BlkUnit *d_bsrc = nullptr, *d_btgt = nullptr;
     const MacItem *d_mitems = nullptr;
@@ -300,7 +301,8 @@ struct sgf_batch {
     // cross-level pairs (plans with block convolutions): their block arguments, per
     // pass the first CTA of every such plan, and the products of all of them, plans
     // that share spectra together
-    int blk_plans = 0, blk_rounds = 0, mac_blocks = 0, mac_items = 0;
+    int blk_plans = 0, blk_rounds = 0;
+    MacLaunch mac;
     int blk_blocks[BLK_PASSES + kMaxStages] = {};  // CTAs of the passes, then of the inverse-row rounds
     void *d_blk = nullptr;
     size_t off_prefix = 0, off_index = 0, off_items = 0, off_terms = 0, off_xo = 0, off_ao = 0;  // in d_blk
@@ -597,37 +599,41 @@ int blk_tw_offset(int logB)
     return o;
 }
 
-// Target units a warp takes: the accumulators (QG targets, two components, R right-hand
-// sides) have to stay in registers.
-int mac_qg(int qg, int rhs) { return std::min(qg, rhs == 1 ? 4 : rhs == 2 ? 2 : 1); }
+// Target units a warp takes: the accumulators (QG targets and their mirror images, two
+// components, R right-hand sides) have to stay in registers.
+int mac_qg(int qg, int rhs, int sym) { return std::min(qg, sym ? 1 : rhs == 1 ? 4 : rhs == 2 ? 2 : 1); }
 
 // Work items of the products: targets whose terms read the same kernel spectra
-// share them, up to four right-hand sides an item (the accumulators of more do
-// not fit in registers).  QG targets per warp (mac_qg): fewer where the launch would leave SMs without warps
-// (16 warps on each of 152 SMs).  Long items first.
+// share them, up to four right-hand sides an item, two where mirror images are summed
+// too (the accumulators of more do not fit in registers).  QG targets per warp
+// (mac_qg): fewer where the launch would leave SMs without warps (16 warps on each
+// of 152 SMs).  Mirror-symmetric items first, long ones before short ones.
 void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &items, std::vector<MacTerm> &terms,
-               std::vector<size_t> &xo, std::vector<size_t> &ao, int *blocks)
+               std::vector<size_t> &xo, std::vector<size_t> &ao, MacLaunch *launch)
 {
     std::map<std::vector<size_t>, std::vector<int>> by_k;
     std::vector<std::vector<size_t>> order;
     for (int i = 0; i < (int)tg.size(); ++i) {
-        std::vector<size_t> key{(size_t)tg[i].m2, (size_t)tg[i].F};
+        std::vector<size_t> key{tg[i].sym ? 1u : 0u, (size_t)tg[i].m2, (size_t)tg[i].F, (size_t)tg[i].sym};
         for (const auto &t : tg[i].terms)
             key.insert(key.end(), {t.k_off, t.sp, t.sq});
         if (!by_k.count(key))
             order.push_back(key);
         by_k[key].push_back(i);
     }
-    std::stable_sort(order.begin(), order.end(),
-                     [](const std::vector<size_t> &x, const std::vector<size_t> &y) { return x[0] > y[0]; });
+    std::stable_sort(order.begin(), order.end(), [](const std::vector<size_t> &x, const std::vector<size_t> &y) {
+        return x[0] != y[0] ? x[0] > y[0] : x[1] > y[1];
+    });
     items.clear();
     terms.clear();
     xo.clear();
     ao.clear();
+    *launch = MacLaunch{};
     for (const auto &key : order) {
         const auto &v = by_k[key];
-        for (size_t b = 0; b < v.size(); b += 4) {
-            const int R = (int)std::min<size_t>(4, v.size() - b);
+        const size_t most = key[0] ? 2 : 4;
+        for (size_t b = 0; b < v.size(); b += most) {
+            const int R = (int)std::min<size_t>(most, v.size() - b);
             const BlkTarget &t0 = tg[v[b]];
             MacItem it{};
             it.term_begin = (int)terms.size();
@@ -636,6 +642,9 @@ void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &
             it.rhs = R;
             it.m2 = t0.m2;
             it.F = t0.F;
+            it.logm = t0.logm;
+            it.logB = t0.logB;
+            it.sym = t0.sym;
             for (size_t k = 0; k < t0.terms.size(); ++k) {
                 terms.push_back(MacTerm{t0.terms[k].k_off, t0.terms[k].sp, t0.terms[k].sq, (int)xo.size(), 0});
                 for (int r = 0; r < R; ++r)
@@ -643,27 +652,31 @@ void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &
             }
             for (int r = 0; r < R; ++r)
                 ao.push_back(tg[v[b + r]].a_off);
-            it.tiles = (it.F / vec + 31) / 32;
+            // a lane's frequencies: 16 bytes of them, or one and its mirror
+            it.tiles = ((it.sym ? ((1 << it.logB) + 1) * ((1 << it.logB) + 1) : it.F / vec) + 31) / 32;
             items.push_back(it);
         }
     }
+    auto units = [](const MacItem &it) {  // target units the warps run over
+        return it.m2 >> ((it.sym & kMirrorX ? 1 : 0) + (it.sym & kMirrorY ? 1 : 0));
+    };
     int qg = 4;
     for (; qg > 1; qg >>= 1) {
         long long warps = 0;
         for (const auto &it : items)
-            warps += (long long)it.tiles * (it.m2 / mac_qg(qg, it.rhs));
+            warps += (long long)it.tiles * std::max(1, units(it) / mac_qg(qg, it.rhs, it.sym));
         if (warps >= 16 * 152)
             break;
     }
-    int blk = 0;
     for (auto &it : items) {
-        it.qg = mac_qg(qg, it.rhs);
-        it.nqg = it.m2 / it.qg;
+        it.qg = std::min(units(it), mac_qg(qg, it.rhs, it.sym));
+        it.nqg = units(it) / it.qg;
+        int &blk = it.sym ? launch->sym_blocks : launch->blocks;
+        (it.sym ? launch->sym_items : launch->items)++;
         it.blk_begin = blk;
         const long long warps = (long long)it.tiles * it.nqg;
         blk += (int)((warps + kBlkThreads / 32 - 1) / (kBlkThreads / 32));
     }
-    *blocks = blk;
 }
 
 // The stages, sources, targets and products of a plan's cross-level pairs; off:
@@ -673,7 +686,8 @@ void build_blocks(sgf_plan *p, size_t off)
 {
     const Forest &fo = p->fo;
     const size_t Cb = 2 * p->esize;
-    std::map<SetKey, int> group;  // first set of a pair's m^2 phases
+    std::map<SetKey, int> group;    // first set of a pair's m^2 phases
+    std::map<int, int> group_sym;   // mirror symmetry that all targets reading it have
     auto get_group = [&](int cas, int m, int ax, int ay, int fine) {
         SetKey key{cas, m, 0, 0, ax, ay, p->pot ? fine : 0};
         auto it = group.find(key);
@@ -696,6 +710,7 @@ void build_blocks(sgf_plan *p, size_t off)
                 p->sets.push_back(g);
             }
         group[key] = first;
+        group_sym[first] = kMirrorX | kMirrorY;
         return first;
     };
     const int nc = p->pot ? 1 : 2;
@@ -727,18 +742,28 @@ void build_blocks(sgf_plan *p, size_t off)
                     bt.a_off = acc;
                     bt.m2 = (int)m2;
                     bt.F = (int)F;
+                    bt.logm = d;
+                    bt.logB = sg.logB;
+                    std::vector<int> first_sets;
                     for (int s = 0; s < fo.K; ++s) {
                         if (fo.level[s] != fo.level[t] + (kind == 0 ? d : -d))
                             continue;
                         const int fi = kind == 0 ? s : t, co = kind == 0 ? t : s;  // finer, coarser
-                        const int g = get_group(kind == 0 ? kBlkCase2 : kBlkCase3, sg.m, fo.org[fi][0] - fo.org[co][0] * sg.m,
-                                                fo.org[fi][1] - fo.org[co][1] * sg.m, fo.level[fi]);
+                        const int ax = fo.org[fi][0] - fo.org[co][0] * sg.m, ay = fo.org[fi][1] - fo.org[co][1] * sg.m;
+                        const int centred = p->N / 2 * (sg.m - 1);  // corner of a patch centred in the coarser one
+                        bt.sym &= p->esize == 8 ? 0 : (ax == centred ? kMirrorX : 0) | (ay == centred ? kMirrorY : 0);
+                        const int g = get_group(kind == 0 ? kBlkCase2 : kBlkCase3, sg.m, ax, ay, fo.level[fi]);
                         const GenSet &g0 = p->sets[g];
                         const size_t per_set = set_bytes_of(p, g0) / Cb, per_blk = (size_t)spec_tables(g0.kind) * F;
                         // set = phase (source of Case 2, target of Case 3), block = the other side
+                        first_sets.push_back(g);
                         bt.terms.push_back({g0.spec_off, kind == 0 ? per_set : per_blk, kind == 0 ? per_blk : per_set,
                                             x_of[kind][s]});
                     }
+                    if (bt.terms.size() > 1)  // several sources: few share a symmetry (eight tiles: 333 us with, 324 without)
+                        bt.sym = 0;
+                    for (int g : first_sets)
+                        group_sym[g] &= bt.sym;
                     acc += nc * m2 * F;
                     p->btgt.push_back(BlkUnit{t, kind});
                     sg.tgt_count[kind]++;
@@ -746,9 +771,12 @@ void build_blocks(sgf_plan *p, size_t off)
                 }
         p->stages.push_back(sg);
     }
+    for (const auto &gs : group_sym)
+        for (int k = gs.first, m2 = p->sets[k].m * p->sets[k].m; k < gs.first + m2; ++k)
+            p->sets[k].cas |= gs.second << kBlkSymShift;
     p->blk_x_elems = x;
     p->blk_elems = x + acc;
-    build_mac(p->btargets, p->esize == 8 ? 1 : 2, p->mitems, p->mterms, p->mxo, p->mao, &p->mac_blocks);
+    build_mac(p->btargets, p->esize == 8 ? 1 : 2, p->mitems, p->mterms, p->mxo, p->mao, &p->mac);
 }
 
 // Block arguments of a solve whose source and target fields start at `work`.
@@ -802,8 +830,7 @@ cudaError_t launch_blocks(const sgf_plan *p, const SolveArgs<T> &a, void *work, 
     cudaError_t e;
     if ((e = pass(BLK_ROWS)) != cudaSuccess || (e = pass(BLK_COLS)) != cudaSuccess)
         return e;
-    if ((e = launch_blk_mac<T>(p->mac_blocks, p->d_mitems, (int)p->mitems.size(), p->d_mterms, p->d_mxo, p->d_mao,
-                               p->spec->dev, k.x, k.acc, a.ncomp, st)) != cudaSuccess)
+    if ((e = launch_blk_mac<T>(p->mac, p->d_mitems, p->d_mterms, p->d_mxo, p->d_mao, p->spec->dev, k.x, k.acc, a.ncomp, st)) != cudaSuccess)
         return e;
     if ((e = pass(BLK_ICOLS)) != cudaSuccess)
         return e;
@@ -1071,7 +1098,7 @@ void reset_lists(sgf_plan *p)
     p->mxo.clear();
     p->mao.clear();
     p->partial_elems = p->fwd_elems = p->bwd_elems = p->blk_x_elems = p->blk_elems = 0;
-    p->mac_blocks = 0;
+    p->mac = MacLaunch{};
 }
 
 // A plan whose kernel spectra exceed its budget.  Residency: the sets of the
@@ -2148,8 +2175,8 @@ sgf_status batch_launches(sgf_batch *bt, cudaStream_t st)
                                             prefix + (size_t)(ps + round) * (bt->blk_plans + 1), index, args, dk, st);
         };
         if ((e = pass(BLK_ROWS)) != cudaSuccess || (e = pass(BLK_COLS)) != cudaSuccess ||
-            (e = launch_blk_mac<T>(bt->mac_blocks, reinterpret_cast<const MacItem *>(base + bt->off_items),
-                                   bt->mac_items, reinterpret_cast<const MacTerm *>(base + bt->off_terms),
+            (e = launch_blk_mac<T>(bt->mac, reinterpret_cast<const MacItem *>(base + bt->off_items),
+                                   reinterpret_cast<const MacTerm *>(base + bt->off_terms),
                                    reinterpret_cast<const size_t *>(base + bt->off_xo),
                                    reinterpret_cast<const size_t *>(base + bt->off_ao), static_cast<const C *>(nullptr),
                                    static_cast<const C *>(nullptr), static_cast<C *>(nullptr), 2, st)) != cudaSuccess ||
@@ -2208,9 +2235,8 @@ sgf_status batch_build_blocks(sgf_batch *bt)
     std::vector<MacItem> items;
     std::vector<MacTerm> terms;
     std::vector<size_t> xo, ao;
-    build_mac(targets, 16 / (int)sizeof(C), items, terms, xo, ao, &bt->mac_blocks);
-    bt->mac_items = (int)items.size();
-    bt->launches++;
+    build_mac(targets, 16 / (int)sizeof(C), items, terms, xo, ao, &bt->mac);
+    bt->launches += (bt->mac.sym_blocks > 0 ? 1 : 0) + (bt->mac.blocks > 0 ? 1 : 0);
     std::vector<unsigned char> blob;
     align_push(blob, args);
     bt->off_prefix = align_push(blob, prefix);
@@ -2956,7 +2982,8 @@ sgf_status sgf_plan_stats_get(const sgf_plan *p, sgf_plan_stats *st)
     st->launches_per_solve = p->restricted + 3 + (p->L > p->fo.R && p->sched.row_inv0 != 1 ? 1 : 0) +
                              (!p->groups.empty() && p->sched.col_case3 == 0 ? 1 : 0) +  // + k_col_g
                              (p->sums.empty() ? 0 : 1) +                                 // + k_col_sum
-                             (p->blk ? 4 + p->fo.depth - 1 : 0);  // + the block passes
+                             (p->blk ? 3 + p->fo.depth - 1 : 0) +  // + the block passes
+                             (p->mac.sym_blocks > 0 ? 1 : 0) + (p->mac.blocks > 0 ? 1 : 0);
     if (p->streamed) {  // column passes: one per non-empty pass; three generator kernels per streamed set
         int passes = 0, streamed_sets = 0;
         for (int ph = 0; ph <= p->waves; ++ph)

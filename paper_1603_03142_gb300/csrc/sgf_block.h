@@ -59,11 +59,22 @@ struct MacItem {
     int term_begin, term_count, a_begin, rhs;
     int m2, F, qg, nqg;       // units, frequencies, targets per warp, target groups
     int tiles, blk_begin;     // frequency tiles of a warp; the item's first CTA
+    int logm, logB, sym, pad; // sym: mirror symmetry of the pairs (kMirrorX | kMirrorY)
 };
 
-// GenSet::cas of a set stored as the m^2 blocks of a block convolution (Case 2, Case 3).
-constexpr int kBlkCase2 = 5, kBlkCase3 = 6;
-inline __host__ __device__ bool gen_blk(const GenSet &g) { return g.cas == kBlkCase2 || g.cas == kBlkCase3; }
+// A pair whose finer patch is centred in the coarser one along an axis (A = N (m - 1)/2)
+// has mirror-symmetric kernels on that axis: the block (p, q) with both units mirrored is the
+// block itself at the mirrored offsets, up to each table's parity.
+enum : int { kMirrorX = 1, kMirrorY = 2 };
+
+// GenSet::cas of a set stored as the m^2 blocks of a block convolution (Case 2, Case 3),
+// and above it the mirror symmetry every use of the set has: the products then read the
+// lower half of the target units in the mirrored axes alone, and the other blocks of a
+// Case 2 set (the whole set of such a phase in Case 3) are not generated.
+constexpr int kBlkCase2 = 5, kBlkCase3 = 6, kBlkSymShift = 4;
+inline __host__ __device__ int gen_case(const GenSet &g) { return g.cas & ((1 << kBlkSymShift) - 1); }
+inline __host__ __device__ int gen_sym(const GenSet &g) { return g.cas >> kBlkSymShift; }
+inline __host__ __device__ bool gen_blk(const GenSet &g) { return gen_case(g) == kBlkCase2 || gen_case(g) == kBlkCase3; }
 
 // A pass of the block convolutions.  Single solve: a, k by value (plans = 1, prefix NULL);
 // batch: da, dk on the device, `plans` of them, prefix[pass] on the device.
@@ -73,10 +84,14 @@ cudaError_t launch_blk_pass(int pass, int round, int blocks, const SolveArgs<T> 
 template <typename T>
 cudaError_t launch_blk_pass_batch(int pass, int round, int blocks, int plans, const int *prefix,
                                   const int *index, const SolveArgs<T> *da, const BlkArgs<T> *dk, cudaStream_t st);
-// The products of `items` work items (blocks CTAs): spec, x and acc are the bases of the
-// offsets (batches: x and acc NULL, the offsets whole addresses / sizeof(complex)).
+// The products: first sym_items mirror-symmetric work items (sym_blocks CTAs), then items
+// (blocks CTAs); spec, x and acc are the bases of the offsets (batches: NULL, the offsets
+// whole addresses / sizeof(complex)).
+struct MacLaunch {
+    int sym_items = 0, sym_blocks = 0, items = 0, blocks = 0;
+};
 template <typename T>
-cudaError_t launch_blk_mac(int blocks, const MacItem *items, int nitems, const MacTerm *terms, const size_t *xo,
+cudaError_t launch_blk_mac(const MacLaunch &l, const MacItem *items, const MacTerm *terms, const size_t *xo,
                            const size_t *ao, const void *spec, const void *x, void *acc, int ncomp, cudaStream_t st);
 // Kernel attributes of the block passes (plan creation).
 template <typename T>

@@ -216,14 +216,17 @@ __global__ void k_gen_tables(GenSet g, int N, double *__restrict__ tables)
 // tables[t][qy m + qx][2B][2B], the convolution indices d in [-(B-1), B-1] of
 // a block and a phase, i.e. D = qB + d (Case 2, target blocks) or d - qB
 // (Case 3, source blocks) in the indexing of Cases 2 and 3 above.
-__global__ void k_gen_tables_blk(GenSet g, int B, double *__restrict__ tables)
+// Generated block i of a set of `bx` blocks a row: its place among the m x m.
+__device__ __forceinline__ int gen_block(int i, int bx, int m) { return (i / bx) * m + i % bx; }
+
+__global__ void k_gen_tables_blk(GenSet g, int B, int bx, double *__restrict__ tables)
 {
     const int P = 2 * B, at = blockIdx.x * blockDim.x + threadIdx.x;
-    const int blk = blockIdx.y, m2 = g.m * g.m;
+    const int blk = gen_block(blockIdx.y, bx, g.m), nb = gridDim.y;
     if (at >= P * P)
         return;
     const int py = at / P, px = at - py * P;
-    const int cas = g.cas == kBlkCase2 ? 2 : 3;
+    const int cas = gen_case(g) == kBlkCase2 ? 2 : 3;
     const AxisMap mx{cas, g.m, g.px, g.ax, B * g.m}, my{cas, g.m, g.py, g.ay, B * g.m};
     double out[6] = {0, 0, 0, 0, 0, 0};
     if (px != B && py != B) {
@@ -237,7 +240,7 @@ __global__ void k_gen_tables_blk(GenSet g, int B, double *__restrict__ tables)
     }
     const int ntab = spec_tables(g.kind);
     for (int t = 0; t < ntab; ++t)
-        tables[((size_t)t * m2 + blk) * P * P + at] = out[t];
+        tables[((size_t)t * nb + blockIdx.y) * P * P + at] = out[t];
 }
 
 // Rows of the P x P tables -> half spectra along x: half[t][kx 0..N][y 0..P)
@@ -272,11 +275,11 @@ __global__ void k_gen_rows(int N, int logN, const double *__restrict__ tables,
 }
 
 // Columns kx of the half spectra -> the stored kernel spectra (scaled by 1/P^2).
-// blocks > 0: a set of block convolutions, table t / blocks of block t % blocks,
-// stored [block][table][kx][ky parity][ky / 2].
+// blocks > 0: generated blocks of a set of block convolutions, table t / blocks of
+// block t % blocks (see gen_block), stored [block][table][kx][ky parity][ky / 2].
 template <typename T>
 __global__ void k_gen_cols(int N, int logN, const double2 *__restrict__ half, const double2 *__restrict__ tw,
-                           int kind, int blocks, void *spec, size_t spec_off)
+                           int kind, int blocks, int bx, int m, void *spec, size_t spec_off)
 {
     using C = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -293,7 +296,7 @@ __global__ void k_gen_cols(int N, int logN, const double2 *__restrict__ half, co
     block_fft<double2, false>(W, N, logN, 2, tw);
     const double scale = 1.0 / ((double)P * (double)P);
     if (blocks > 0) {
-        const int tab = t / blocks, blk = t - tab * blocks, nt_all = gridDim.x / blocks;
+        const int tab = t / blocks, blk = gen_block(t - tab * blocks, bx, m), nt_all = gridDim.x / blocks;
         C *dst = reinterpret_cast<C *>(spec) + spec_off + (((size_t)blk * nt_all + tab) * (N + 1) + kx) * P;
         for (int i = tid; i < P; i += nt) {  // the transform's halves are the ky parities
             C v;
@@ -353,9 +356,13 @@ cudaError_t launch_gen_set(const GenSet &g, int N, int logN, const double2 *tw64
 {
     const int P = 2 * N;
     if (gen_blk(g)) {
-        const int B = N / g.m, m2 = g.m * g.m, nt = spec_tables(g.kind);
+        const bool sx = (gen_sym(g) & kMirrorX) != 0, sy = (gen_sym(g) & kMirrorY) != 0, c2 = gen_case(g) == kBlkCase2;
+        if (!c2 && ((sx && g.px >= g.m / 2) || (sy && g.py >= g.m / 2)))
+            return cudaSuccess;  // a mirror image of another phase's set
+        const int bx = c2 && sx ? g.m / 2 : g.m, by = c2 && sy ? g.m / 2 : g.m;
+        const int B = N / g.m, m2 = bx * by, nt = spec_tables(g.kind);
         const double2 *twb = tw64 + 2 * P - 2 * P / g.m;  // W_2B^k, after the larger tables
-        k_gen_tables_blk<<<dim3((4 * B * B + 255) / 256, m2), 256, 0, st>>>(g, B, work_tables);
+        k_gen_tables_blk<<<dim3((4 * B * B + 255) / 256, m2), 256, 0, st>>>(g, B, bx, work_tables);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
@@ -366,8 +373,8 @@ cudaError_t launch_gen_set(const GenSet &g, int N, int logN, const double2 *tw64
         k_gen_rows<<<dim3(nt * m2, B), gen_threads(B), smem, st>>>(B, logB, work_tables, work_half, twb);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
-        k_gen_cols<T><<<dim3(nt * m2, B + 1), gen_threads(B), smem, st>>>(B, logB, work_half, twb, g.kind, m2, spec,
-                                                                        g.spec_off);
+        k_gen_cols<T><<<dim3(nt * m2, B + 1), gen_threads(B), smem, st>>>(B, logB, work_half, twb, g.kind, m2, bx, g.m,
+                                                                        spec, g.spec_off);
         return cudaGetLastError();
     }
     {
@@ -383,7 +390,7 @@ cudaError_t launch_gen_set(const GenSet &g, int N, int logN, const double2 *tw64
     k_gen_rows<<<dim3(ntab, P / 2), gen_threads(N), smem, st>>>(N, logN, work_tables, work_half, tw64);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    k_gen_cols<T><<<dim3(ntab, N + 1), gen_threads(N), smem, st>>>(N, logN, work_half, tw64, g.kind, 0, spec,
+    k_gen_cols<T><<<dim3(ntab, N + 1), gen_threads(N), smem, st>>>(N, logN, work_half, tw64, g.kind, 0, 1, 1, spec,
                                                                      g.spec_off);
     return cudaGetLastError();
 }

@@ -65,3 +65,35 @@ def test_blocks_equal_the_direct_sum(case, m, N, ax, ay):
     ref = _direct(case, m, N, ax, ay, s)
     # N^2 terms of order one, transforms of at most 2N points a side
     assert np.abs(_blocks(case, m, N, ax, ay, s) - ref).max() <= 64 * np.finfo(float).eps * N * N
+
+
+@pytest.mark.parametrize("case", [2, 3])
+@pytest.mark.parametrize("m,N", [(2, 8), (4, 16)])
+@pytest.mark.parametrize("mx,my", [(True, False), (False, True), (True, True)])
+def test_centred_pairs_are_mirror_images(case, m, N, mx, my):
+    """A finer patch centred in the coarser one (A = N (m - 1)/2): the block of mirrored units
+    is the block at the mirrored offsets, which per frequency is the value at -ky (y mirrored),
+    its conjugate there (x mirrored) or its own conjugate (both), for a table even in both axes."""
+    B, P, A = N // m, 2 * (N // m), N * (m - 1) // 2
+    d = np.arange(P)
+    d = np.where(d < B, d, d - P)
+    live = np.arange(P) != B
+
+    def edge(ph, blk):  # lower edge of the source cell, target centre at 0
+        D = blk * B + d if case == 2 else d - blk * B
+        return -m * D + ph - 0.5 * m + A if case == 2 else -m * D - ph - A - 0.5
+
+    w = 1.0 if case == 2 else float(m)
+
+    def block(p, q):  # p, q = (x, y): phase and block of Case 2, block and phase of Case 3
+        ph, bl = (p, q) if case == 2 else (q, p)
+        u, v = edge(ph[0], bl[0])[None, :] + 0.5 * w, edge(ph[1], bl[1])[:, None] + 0.5 * w
+        return np.fft.fft2(np.where(live[None, :] & live[:, None], np.cos(0.3 * u) * np.exp(-0.01 * v * v), 0.0))
+
+    back = -np.arange(P)
+    for p in [(x, y) for x in range(m) for y in range(m)]:
+        for q in [(x, y) for x in range(m) for y in range(m)]:
+            mir = lambda a: (m - 1 - a[0] if mx else a[0], m - 1 - a[1] if my else a[1])
+            K = block(p, q)
+            want = K[back] if my and not mx else np.conj(K[back]) if mx and not my else np.conj(K)
+            assert np.abs(block(mir(p), mir(q)) - want).max() <= 1e-12 * max(1.0, np.abs(K).max())

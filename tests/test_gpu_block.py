@@ -54,6 +54,9 @@ NESTS = {
     "512x2_corner": (W.Nest(n=512, levels=2, off=[(0, 0), (0, 256)]), ("fp32", "bf16x")),
     "256x3_odd": (W.Nest(n=256, levels=3, off=[(0, 0), (37, 90), (101, 3)]), ("fp32", "bf16x")),
     "256x5": (W.Nest(n=256, levels=5, off=[(0, 0), (64, 65), (63, 7), (128, 64), (31, 33)]), ("fp32",)),
+    "256x3_centred": (W.centred_nest(256, 3), ("fp32",)),       # mirror-symmetric pairs in both axes
+    "256x4_mirror_y": (W.centred_nest(256, 4, centre=(0.3, 0.0)), ("fp32",)),
+    "512x3_mirror_x": (W.centred_nest(512, 3, centre=(0.0, -0.2)), ("fp32", "bf16x")),
     "300x3_embedded": (W.Nest(n=300, levels=3, off=[(0, 0), (75, 11), (150, 80)]), ("fp32",)),
     "1024x4": (W.Nest(n=1024, levels=4, off=[(0, 0), (255, 256), (301, 4), (256, 511)]), ("fp32",)),
     "2048x2": (W.Nest(n=2048, levels=2, off=[(0, 0), (513, 700)]), ("fp32",)),
@@ -75,7 +78,8 @@ def test_block_pairs_against_oracle(lib, name, prec):
     assert _worst(geom, (gx, gy), (ox, oy), samp) <= tol(prec, geom.n)
 
 
-@pytest.mark.parametrize("name", ["512x2_corner", "256x3_odd", "256x5", "300x3_embedded"])
+@pytest.mark.parametrize("name", ["512x2_corner", "256x3_odd", "256x5", "300x3_embedded", "256x3_centred",
+                                  "256x4_mirror_y", "512x3_mirror_x"])
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_block_pairs_equal_whole_grid_pairs(lib, name, prec):
     """A plan over its spectra budget runs the whole-grid passes on the same FP64 tables: the
@@ -94,9 +98,10 @@ def test_block_pairs_equal_whole_grid_pairs(lib, name, prec):
         assert d <= 256 * eps * scale, (l, d / scale)
 
 
-@pytest.mark.parametrize("prec", ["fp32"])
-def test_block_potential_against_oracle(lib, prec):
-    geom = NESTS["256x3_odd"][0]
+@pytest.mark.parametrize("name,prec", [("256x3_odd", "fp32"), ("256x3_centred", "fp32"), ("256x4_mirror_y", "fp32"),
+                                       ("512x3_mirror_x", "fp32")])
+def test_block_potential_against_oracle(lib, name, prec):
+    geom = NESTS[name][0]
     sigma = _sigma(geom, 4)
     plan = lib.Plan(geom, prec, potential=True)
     dt = torch.float64 if prec == "fp64" else torch.float32

@@ -135,6 +135,13 @@ struct KShape {
     static constexpr int N = 1 << LOGN, V = !TC && N <= kSlot4Max ? 4 : 16, Q = N / V;
     static constexpr int ROW_THREADS = 2 * Q < 32 ? 32 : 2 * Q;  // both parity halves
     static constexpr int COL_THREADS = Q < 32 ? 32 : Q;          // one parity half
+    // Columns a CTA of the cluster column kernels (k_col, k_col_g, k_col_sum) takes side by side.
+    // A tensor-core tile has 128 rows, one per slot, and a stage waits for one round trip whatever
+    // number of them is filled: one 512-point column fills 32.  Column passes of a 512^2 nest of 4
+    // levels in SGF_BF16X, one -> four columns a CTA: 8.1 -> 4.4 ms; 1024^2 3 levels, two columns:
+    // 5.4 -> 3.9; 256^2 3 levels, eight: 0.80 -> 0.32.
+    static constexpr int CPC = !TC || Q >= 128 ? 1 : 128 / Q < 8 ? 128 / Q : 8;
+    static constexpr int CG_THREADS = CPC * Q < 32 ? 32 : CPC * Q;
     static constexpr int SP_ROW = N + N / 16 + 8;  // pad puts the two halves 16 banks apart for the unpack
     // threads per parity half for the half barriers of the row kernels (0: whole-block barriers)
     static constexpr int HB_ROW = V == 16 && Q >= 32 ? Q : 0;
@@ -159,7 +166,10 @@ enum : int {
 };
 __host__ __device__ constexpr int tc_round(int logn, int tiles, int kind)
 {
-    return logn < 12                                 ? tiles
+    // k_col_g with 128 slots a CTA (N = 256 .. 1024): one buffer for its two tiles leaves room for a
+    // second CTA on the SM, worth more than the second round of its dual inverse transforms (column
+    // passes of a 512^2 nest of 4 levels through it 7.5 -> 4.9 ms, 1024^2 3 levels 6.8 -> 4.7)
+    return logn < 12 ? (kind == KK_COL_G && logn >= 8 && logn <= 10 ? 1 : tiles)
            : kind == KK_ROW_FWD                      ? (tiles < 2 ? tiles : 2)
            : kind == KK_ROW_INV || kind == KK_COL_G || kind == KK_ROW_INV2 || kind == KK_COL_MW ? 1
                                                                           : tiles;
@@ -417,7 +427,7 @@ struct ColStage {
 // the fold of the odd half reuses them afterwards.
 constexpr int kColWalk = 4;
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG_THREADS) k_col(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
@@ -426,7 +436,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     constexpr int N = K::N, Q = K::Q, P = 2 * N, QS = quarter_stride(N), HQ = quarter_half(N);
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::CG_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -435,7 +445,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
         tc_begin(tcx, smem_tc, TCT, TCR, a.status, a.wait_cycles, a.inject);
     C *tw = reinterpret_cast<C *>(smem_raw);
     C *sbuf = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));
-    unsigned char *stage_base = reinterpret_cast<unsigned char *>(sbuf + SPC);
+    unsigned char *stage_base = reinterpret_cast<unsigned char *>(sbuf + K::CPC * SPC);
     using CS = ColStage<T, LOGN, TC>;
     constexpr size_t stage_bytes = CS::BYTES;
     cg::cluster_group cluster = cg::this_cluster();
@@ -443,19 +453,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     const ColWork w = a.col_list[wm.y];
     const ColOutput o = a.outs[w.out];
     const int t = threadIdx.x;
-    const bool active = t < Q;
-    const int j = active ? t : 0;
+    constexpr int CPC = K::CPC;
+    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
     const int nitems = 3 * w.in_count;
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     cp_block(tw, a.tw, tw_bytes<C>(a.tw_entries));
     // tensor-core instances: a cluster takes kColWalk columns of its work item, gridDim.x / 2
     // apart (the tiles, the tensor memory and the twiddles set up once for them)
     constexpr bool WALK = TC && !BATCH;
-    for (int kx = blockIdx.x >> 1; kx <= N; kx += WALK ? (int)(gridDim.x >> 1) : N + 1) {
-        if (WALK && kx != (int)(blockIdx.x >> 1))
-            __syncthreads();  // the previous column's fold (over sbuf and the stages) has been read
-        auto issue = [&](int k) {
-            unsigned char *st = stage_base + (size_t)(k & 1) * stage_bytes;
+    const int kx_first = (int)(blockIdx.x >> 1) * CPC;
+    for (int kx0 = kx_first; kx0 <= N; kx0 += WALK ? (int)(gridDim.x >> 1) * CPC : N + 1) {
+        const int kx = kx0 + c;
+        const bool active = t < CPC * Q && kx <= N;
+        if (WALK && kx0 != kx_first)
+            __syncthreads();  // the previous columns' folds (over sbuf and the stages) have been read
+        auto issue_col = [&](int k, int cc) {
+            const int kx = kx0 + cc;
+            unsigned char *st = stage_base + (size_t)((k & 1) * CPC + cc) * stage_bytes;
             const ColInput ci = a.ins[w.in_begin + k / 3];
             const FwdSlab sl = a.slabs[ci.slab];
             const int f = k % 3;
@@ -478,6 +492,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
                 }
             }
         };
+        auto issue = [&](int k) {
+            for (int cc = 0; cc < CPC && kx0 + cc <= N; ++cc)
+                issue_col(k, cc);
+        };
         issue(0);
         cp_commit();
         if (nitems > 1)
@@ -493,7 +511,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
         for (int k = 0; k < nitems; ++k) {
             cp_wait<1>();
             __syncthreads();
-            const unsigned char *st = stage_base + (size_t)(k & 1) * stage_bytes;
+            const unsigned char *st = stage_base + (size_t)((k & 1) * CPC + c) * stage_bytes;
             const C *col = reinterpret_cast<const C *>(st);
             const T *spx = reinterpret_cast<const T *>(st + (size_t)N * sizeof(C));
             const ColInput ci = a.ins[w.in_begin + k / 3];
@@ -513,7 +531,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
                     v[0][u] = x;
                 }
             }
-            fft_ct<C, false, LOGN, 1, TC>(v, sbuf, SPC, j, active, tw, &tcx);
+            fft_ct<C, false, LOGN, 1, TC>(v, sbuf + c * SPC, SPC, j, active, tw, &tcx);
             if (active) {
                 if (ci.kind == SPEC_QUARTER) {
                     // K0x, K0y imaginary (stored Im), the rest real; bins above N read the
@@ -604,10 +622,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
         // component alone); y[n] = even[n] + W_P^{-n} odd[n]
         const bool two = a.ncomp == 2;
         if (two)
-            fft_ct<C, true, LOGN, 2, TC>(acc, sbuf, SPC, j, active, tw, &tcx);
+            fft_ct<C, true, LOGN, 2, TC>(acc, sbuf + c * 2 * SPC, SPC, j, active, tw, &tcx);
         else
-            fft_ct<C, true, LOGN, 1, TC>(acc, sbuf, SPC, j, active, tw, &tcx);
-        C *fold = sbuf;  // 2N complex over sbuf and the stages
+            fft_ct<C, true, LOGN, 1, TC>(acc, sbuf + c * 2 * SPC, SPC, j, active, tw, &tcx);
+        C *fold = sbuf + c * 2 * N;  // 2N complex a column, over sbuf and the stages
         cluster.sync();
         if (b == 1 && active) {
             C *dst = cluster.map_shared_rank(fold, 0);
@@ -892,7 +910,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, QO ? 512 / KShape<L
 // memory.  Shared memory: twiddle area | sbuf[2 SPC] (the two exchange buffers,
 // then the 2N fold) | fld[3][N].
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col_g(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG_THREADS) k_col_g(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
@@ -901,7 +919,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     constexpr int N = K::N, Q = K::Q, P = 2 * N;
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::CG_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_G);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -909,14 +927,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     if constexpr (TC)
         tc_begin(tcx, smem_tc, TCT, TCR, a.status, a.wait_cycles, a.inject);
     C *tw = reinterpret_cast<C *>(smem_raw);
-    C *sbuf = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));
-    C *fld = sbuf + 2 * SPC;  // after the two exchange buffers of the dual inverse
+    C *sbuf0 = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));  // two exchange buffers a column
     cg::cluster_group cluster = cg::this_cluster();
     const int b = (int)cluster.block_rank();
-    const int kx = blockIdx.x >> 1;
     const int t = threadIdx.x;
-    const bool active = t < Q;
-    const int j = active ? t : 0;
+    constexpr int CPC = K::CPC;
+    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
+    const int kx = (int)(blockIdx.x >> 1) * CPC + c;
+    const bool active = t < CPC * Q && kx <= N;
+    C *sbuf = sbuf0 + c * 2 * SPC;
+    C *fld = sbuf0 + CPC * 2 * SPC + c * 3 * N;  // after the two exchange buffers of the dual inverse
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     const ColGroup g = a.groups[wm.y];
     const FwdSlab sl = a.slabs[a.ins[a.outs[g.out_begin].in_begin].slab];
@@ -1143,7 +1163,7 @@ __global__ void __launch_bounds__(KShape<LOGN>::ROW_THREADS, 1) k_col_gw(SolveAr
 // in k_col.  Shared memory: twiddle area | two exchange buffers (dual inverse),
 // reused for the fold.
 template <typename T, int LOGN, bool BATCH, bool TC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::COL_THREADS) k_col_sum(SolveArgs<T> a0, BatchView<T> bv)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG_THREADS) k_col_sum(SolveArgs<T> a0, BatchView<T> bv)
 {
     const int2 wm = BATCH ? bv.map[blockIdx.y] : make_int2(0, (int)blockIdx.y);
     const SolveArgs<T> &a = BATCH ? bv.args[wm.x] : a0;
@@ -1152,7 +1172,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     constexpr int N = K::N, Q = K::Q;
     constexpr int SPC = col_sp<C>(N);
     extern __shared__ __align__(16) unsigned char smem_tc[];
-    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::COL_THREADS, 2);
+    constexpr int TCT = tc_tiles(KShape<LOGN, TC>::CG_THREADS, 2);
     constexpr int TCR = tc_round(LOGN, TCT, KK_COL_SUM);
     static_assert(!TC || sizeof(T) == 4, "tensor-core tiles take FP32 data");
     unsigned char *smem_raw = smem_tc + (TC ? tc_smem_bytes(TCR) : 0);
@@ -1160,13 +1180,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CO
     if constexpr (TC)
         tc_begin(tcx, smem_tc, TCT, TCR, a.status, a.wait_cycles, a.inject);
     C *tw = reinterpret_cast<C *>(smem_raw);
-    C *sbuf = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));
+    C *sbuf0 = reinterpret_cast<C *>(smem_raw + tw_bytes<C>(a.tw_entries));  // two exchange buffers a column
     cg::cluster_group cluster = cg::this_cluster();
     const int b = (int)cluster.block_rank();
-    const int kx = blockIdx.x >> 1;
     const int t = threadIdx.x;
-    const bool active = t < Q;
-    const int j = active ? t : 0;
+    constexpr int CPC = K::CPC;
+    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
+    const int kx = (int)(blockIdx.x >> 1) * CPC + c;
+    const bool active = t < CPC * Q && kx <= N;
+    C *sbuf = sbuf0 + c * 2 * SPC;
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     const ColSum sm = a.sums[wm.y];
     const ColOutput o = a.outs[sm.out];
@@ -2811,9 +2833,11 @@ struct KSmem {
         // the staged rows (at most 4 N reals) fit in the exchange buffers' 2 SP_ROW complex
         return rtc(KK_ROW_FWD) + tw() + 2 * (size_t)KShape<LOGN, TC>::SP_ROW * sizeof(C);
     }
+    static constexpr int CPC = KShape<LOGN, TC>::CPC;
+    static size_t gtc(int kind) { return tc(KShape<LOGN, TC>::CG_THREADS, 2, kind); }
     static size_t col()
     {
-        return ctc(KK_COL) + tw() + (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColStage<T, LOGN, TC>::BYTES;
+        return gtc(KK_COL) + tw() + CPC * ((size_t)col_sp<C>(N) * sizeof(C) + 2 * ColStage<T, LOGN, TC>::BYTES);
     }
     static size_t col_w() { return tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColWStage<T, LOGN, false>::BYTES; }
     static size_t col_wq() { return tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) + 2 * ColWStage<T, LOGN, true>::BYTES; }
@@ -2845,13 +2869,12 @@ struct KSmem {
     }
     static size_t col_g()
     {
-        return tc(KShape<LOGN, TC>::COL_THREADS, 2, KK_COL_G) + tw() + 2 * (size_t)col_sp<C>(N) * sizeof(C) +
-               3 * (size_t)N * sizeof(C);
+        return gtc(KK_COL_G) + tw() + CPC * (2 * (size_t)col_sp<C>(N) * sizeof(C) + 3 * (size_t)N * sizeof(C));
     }
     static size_t col_sum()
     {
         size_t body = 2 * (size_t)col_sp<C>(N) * sizeof(C);  // two exchange buffers; the 2N fold fits
-        return ctc(KK_COL_SUM) + tw() + body;
+        return gtc(KK_COL_SUM) + tw() + CPC * body;
     }
     static size_t col_mw()
     {
@@ -3064,9 +3087,10 @@ cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t
     case PASS_COL: {
         // tensor-core tiles: each cluster walks kColWalk columns of its work item (strided by the
         // clusters of the item), which keeps many clusters per item for balance
-        const int gx = TC && !batch ? 2 * ((K::N + 1 + kColWalk - 1) / kColWalk) : 2 * (K::N + 1);
+        const int walk = TC && !batch ? (kColWalk > K::CPC ? kColWalk / K::CPC : 1) : 1;
+        const int gx = 2 * ((K::N + walk * K::CPC) / (walk * K::CPC));
         SGF_LAUNCH((k_col<T, LOGN, false, TC>), (k_col<T, LOGN, true, TC>), 2, S::col(), dim3(gx, count),
-                   K::COL_THREADS)
+                   K::CG_THREADS)
         break;
     }
     case PASS_ROW_INV: {
@@ -3132,12 +3156,12 @@ cudaError_t launch_pass(int pass, const SolveArgs<T> &a, int count, cudaStream_t
     }
     case PASS_COL_SUM: {
         SGF_LAUNCH((k_col_sum<T, LOGN, false, TC>), (k_col_sum<T, LOGN, true, TC>), 16, S::col_sum(),
-                   dim3(2 * (K::N + 1), count), K::COL_THREADS)
+                   dim3(2 * ((K::N + K::CPC) / K::CPC), count), K::CG_THREADS)
         break;
     }
     case PASS_COL_G: {
         SGF_LAUNCH((k_col_g<T, LOGN, false, TC>), (k_col_g<T, LOGN, true, TC>), 14, S::col_g(),
-                   dim3(2 * (K::N + 1), count), K::COL_THREADS)
+                   dim3(2 * ((K::N + K::CPC) / K::CPC), count), K::CG_THREADS)
         break;
     }
     case PASS_COL_MW: {

@@ -212,6 +212,10 @@ struct sgf_plan {
     std::vector<size_t> mxo, mao;
     MacLaunch mac;
     size_t blk_x_elems = 0, blk_elems = 0;  // complex elements: source fields; source and target fields
+    // blk_beside plans: their passes up to the inverse rows run beside the patches' own on a
+    // stream of the plan, forked from the solve's stream and joined before the inverse rows
+    cudaStream_t side = nullptr;
+    cudaEvent_t side_fork = nullptr, side_join = nullptr;
     const BlkUnit *d_bsrc = nullptr, *d_btgt = nullptr;
     const MacItem *d_mitems = nullptr;
     const MacTerm *d_mterms = nullptr;
@@ -819,25 +823,41 @@ void fill_blk(const sgf_plan *p, void *work, BlkArgs<T> &k)
     k.acc = k.x + p->blk_x_elems;
 }
 
-// The cross-level pairs of a solve, added to the forces (or the potential) that the
-// patches' own passes have stored.
+// The cross-level pairs of a solve up to their inverse rows: needs the (restricted)
+// densities alone.
 template <typename T>
-cudaError_t launch_blocks(const sgf_plan *p, const SolveArgs<T> &a, void *work, cudaStream_t st)
+cudaError_t launch_blocks_sums(const sgf_plan *p, const SolveArgs<T> &a, const BlkArgs<T> &k, cudaStream_t st)
 {
-    BlkArgs<T> k{};
-    fill_blk<T>(p, work, k);
     auto pass = [&](int ps) { return launch_blk_pass<T>(ps, 0, k.blocks[ps][k.stages], a, k, st); };
     cudaError_t e;
     if ((e = pass(BLK_ROWS)) != cudaSuccess || (e = pass(BLK_COLS)) != cudaSuccess)
         return e;
     if ((e = launch_blk_mac<T>(p->mac, p->d_mitems, p->d_mterms, p->d_mxo, p->d_mao, p->spec->dev, k.x, k.acc, a.ncomp, st)) != cudaSuccess)
         return e;
-    if ((e = pass(BLK_ICOLS)) != cudaSuccess)
-        return e;
-    for (int r = 0; r < k.rounds; ++r)
-        if ((e = launch_blk_pass<T>(BLK_IROWS, r, k.seg[r][k.segs[r]].blk, a, k, st)) != cudaSuccess)
+    return pass(BLK_ICOLS);
+}
+
+// Their inverse rows, added to the forces (or the potential) that the patches' own
+// passes have stored.
+template <typename T>
+cudaError_t launch_blocks_add(const SolveArgs<T> &a, const BlkArgs<T> &k, cudaStream_t st)
+{
+    for (int r = 0; r < k.rounds; ++r) {
+        const cudaError_t e = launch_blk_pass<T>(BLK_IROWS, r, k.seg[r][k.segs[r]].blk, a, k, st);
+        if (e != cudaSuccess)
             return e;
+    }
     return cudaSuccess;
+}
+
+// Both, one after the other, with the fields at `work`.
+template <typename T>
+cudaError_t launch_blocks(const sgf_plan *p, const SolveArgs<T> &a, void *work, cudaStream_t st)
+{
+    BlkArgs<T> k{};
+    fill_blk<T>(p, work, k);
+    const cudaError_t e = launch_blocks_sums<T>(p, a, k, st);
+    return e != cudaSuccess ? e : launch_blocks_add<T>(a, k, st);
 }
 
 // Build all host-side lists of a plan (no CUDA calls).  Every ordered pair of
@@ -1276,6 +1296,14 @@ void plan_free_owned(sgf_plan *p)
     if (p->done)
         cudaEventDestroy(p->done);
     p->done = nullptr;
+    for (cudaEvent_t *ev : {&p->side_fork, &p->side_join}) {
+        if (*ev)
+            cudaEventDestroy(*ev);
+        *ev = nullptr;
+    }
+    if (p->side)
+        cudaStreamDestroy(p->side);
+    p->side = nullptr;
     p->d_status = nullptr;
     p->d_lists = p->d_fwd = p->d_bwd = p->d_restricted = p->d_stage = nullptr;
     cudaSetDevice(cur);
@@ -1301,12 +1329,32 @@ size_t io_stage_bytes(const sgf_plan *p)
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Bytes of a solve's intermediates: the forward slabs and behind them the column
-// outputs, and, once the patches' own passes are done with those, the fields of the
-// block convolutions.
-size_t inter_bytes(const sgf_plan *p)
+// outputs; the fields of the block convolutions take their place once the patches' own
+// passes are done with them, or (blk_beside) follow at blk_offset, in single solves
+// that run both at once.  Batches and the no-allocation solve run one after the other
+// in the shared place.
+size_t serial_inter_bytes(const sgf_plan *p)
 {
     const size_t Cb = 2 * p->esize;
     return std::max(align256(p->fwd_elems * Cb) + p->bwd_elems * Cb, p->blk_elems * Cb);
+}
+// Small solves, whose passes leave SMs idle: side by side they take (us, one after the
+// other / beside; centred nests) 256^2 2, 3 and 4 levels 80 / 60, 135 / 109, 245 / 233,
+// 512^2 2 levels 134 / 127.  Larger ones fill the SMs and lose what one part leaves in
+// L2 for the next: 256^2 5 levels 591 / 631, 512^2 3 and 4 levels 298 / 342, 656 / 956,
+// 1024^2 3 levels 968 / 1193.
+bool blk_beside(const sgf_plan *p)
+{
+    return p->blk && (p->N <= 256 ? p->fo.depth <= 4 : p->N <= 512 && p->fo.depth == 2);
+}
+size_t blk_offset(const sgf_plan *p)
+{
+    const size_t Cb = 2 * p->esize;
+    return blk_beside(p) ? align256(p->fwd_elems * Cb) + align256(p->bwd_elems * Cb) : 0;
+}
+size_t inter_bytes(const sgf_plan *p)
+{
+    return blk_beside(p) ? blk_offset(p) + p->blk_elems * 2 * p->esize : serial_inter_bytes(p);
 }
 
 // Device bytes plan_alloc_owned allocates for p (lists, intermediates, restricted densities).
@@ -1449,6 +1497,10 @@ sgf_status plan_alloc_owned(sgf_plan *p)
         return cuda_fail(e, "cudaMemset(status word)");
     if ((e = cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming)) != cudaSuccess)
         return cuda_fail(e, "cudaEventCreate(solve completion)");
+    if (blk_beside(p) && ((e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking)) != cudaSuccess ||
+                   (e = cudaEventCreateWithFlags(&p->side_fork, cudaEventDisableTiming)) != cudaSuccess ||
+                   (e = cudaEventCreateWithFlags(&p->side_join, cudaEventDisableTiming)) != cudaSuccess))
+        return cuda_fail(e, "stream of the block convolutions");
     p->workspace_bytes = workspace_of(p);
     return p->tma_inv ? encode_tmap_inv(p) : SGF_OK;
 }
@@ -1864,6 +1916,15 @@ sgf_status solve_core(sgf_plan *p, const void *const *sigma, void *const *fx, vo
     cudaError_t e;
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
+    BlkArgs<T> blk{};
+    const bool beside = blk_beside(p) && !p->profile;  // timed passes run one after the other
+    if (p->blk)
+        fill_blk<T>(p, static_cast<unsigned char *>(p->d_fwd) + blk_offset(p), blk);
+    if (beside && ((e = cudaEventRecord(p->side_fork, st)) != cudaSuccess ||
+                   (e = cudaStreamWaitEvent(p->side, p->side_fork, 0)) != cudaSuccess ||
+                   (e = launch_blocks_sums<T>(p, a, blk, p->side)) != cudaSuccess ||
+                   (e = cudaEventRecord(p->side_join, p->side)) != cudaSuccess))
+        return cuda_fail(e, "block convolution launch");
     e = p->merged ? launch_pass_n<T>(zero_rim_fwd_pass(p), p->logN, a, 0, st,
                                      nullptr, p->tc)
                   : launch_pass_n<T>(general_fwd_pass(p), p->logN, a, (int)p->items.size(), st, nullptr, p->tc);
@@ -1882,8 +1943,11 @@ sgf_status solve_core(sgf_plan *p, const void *const *sigma, void *const *fx, vo
         return cuda_fail(e, "row_inv launch");
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
-    if (p->blk && (e = launch_blocks<T>(p, a, p->d_fwd, st)) != cudaSuccess)
-        return cuda_fail(e, "block convolution launch");
+    if (p->blk) {
+        e = beside ? cudaStreamWaitEvent(st, p->side_join, 0) : launch_blocks_sums<T>(p, a, blk, st);
+        if (e != cudaSuccess || (e = launch_blocks_add<T>(a, blk, st)) != cudaSuccess)
+            return cuda_fail(e, "block convolution launch");
+    }
     return mark(p, st);
 }
 
@@ -1994,7 +2058,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[SGF_NOALLOC_SCR
 size_t noalloc_bytes(const sgf_plan *p)
 {
     const size_t Cb = 2 * p->esize;
-    return align256((size_t)p->restricted * p->N * p->N * p->esize) + align256(inter_bytes(p)) +
+    return align256((size_t)p->restricted * p->N * p->N * p->esize) + align256(serial_inter_bytes(p)) +
            align256(p->partial_elems * Cb);
 }
 
@@ -2021,7 +2085,7 @@ sgf_status solve_noalloc_impl(sgf_plan *p, const void *const *sigma, void *const
     T *restricted = reinterpret_cast<T *>(scratch);
     unsigned char *fwd = scratch + align256((size_t)p->restricted * N * N * p->esize);
     unsigned char *bwd = fwd + align256(p->fwd_elems * Cb);
-    unsigned char *partial = fwd + align256(inter_bytes(p));
+    unsigned char *partial = fwd + align256(serial_inter_bytes(p));
     SolveArgs<T> a{};
     fill_geometry(p, a);
     cudaError_t er = fill_sources<T>(p, sigma, restricted, a, true, st);

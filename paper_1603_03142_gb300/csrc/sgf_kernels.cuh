@@ -454,7 +454,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG
     const ColOutput o = a.outs[w.out];
     const int t = threadIdx.x;
     constexpr int CPC = K::CPC;
-    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
+    const int c = CPC > 1 && t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
     const int nitems = 3 * w.in_count;
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     cp_block(tw, a.tw, tw_bytes<C>(a.tw_entries));
@@ -464,7 +464,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG
     const int kx_first = (int)(blockIdx.x >> 1) * CPC;
     for (int kx0 = kx_first; kx0 <= N; kx0 += WALK ? (int)(gridDim.x >> 1) * CPC : N + 1) {
         const int kx = kx0 + c;
-        const bool active = t < CPC * Q && kx <= N;
+        const bool active = t < CPC * Q && (CPC == 1 || kx <= N);
         if (WALK && kx0 != kx_first)
             __syncthreads();  // the previous columns' folds (over sbuf and the stages) have been read
         auto issue_col = [&](int k, int cc) {
@@ -932,9 +932,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG
     const int b = (int)cluster.block_rank();
     const int t = threadIdx.x;
     constexpr int CPC = K::CPC;
-    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
+    const int c = CPC > 1 && t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
     const int kx = (int)(blockIdx.x >> 1) * CPC + c;
-    const bool active = t < CPC * Q && kx <= N;
+    const bool active = t < CPC * Q && (CPC == 1 || kx <= N);
     C *sbuf = sbuf0 + c * 2 * SPC;
     C *fld = sbuf0 + CPC * 2 * SPC + c * 3 * N;  // after the two exchange buffers of the dual inverse
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
@@ -1185,9 +1185,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(KShape<LOGN, TC>::CG
     const int b = (int)cluster.block_rank();
     const int t = threadIdx.x;
     constexpr int CPC = K::CPC;
-    const int c = t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
+    const int c = CPC > 1 && t < CPC * Q ? t / Q : 0, j = t < CPC * Q ? t - c * Q : 0;  // this thread's column and slot
     const int kx = (int)(blockIdx.x >> 1) * CPC + c;
-    const bool active = t < CPC * Q && kx <= N;
+    const bool active = t < CPC * Q && (CPC == 1 || kx <= N);
     C *sbuf = sbuf0 + c * 2 * SPC;
     const TwLayout tl = tw_layout(F16<LOGN>::twlen, N);
     const ColSum sm = a.sums[wm.y];

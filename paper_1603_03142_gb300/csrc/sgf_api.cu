@@ -1920,33 +1920,39 @@ sgf_status solve_core(sgf_plan *p, const void *const *sigma, void *const *fx, vo
     const bool beside = blk_beside(p) && !p->profile;  // timed passes run one after the other
     if (p->blk)
         fill_blk<T>(p, static_cast<unsigned char *>(p->d_fwd) + blk_offset(p), blk);
+    // A failed launch leaves st behind what the side stream was given.
+    auto leave = [&](cudaError_t err, const char *what) {
+        if (beside && cudaEventRecord(p->side_join, p->side) == cudaSuccess)
+            cudaStreamWaitEvent(st, p->side_join, 0);
+        return cuda_fail(err, what);
+    };
     if (beside && ((e = cudaEventRecord(p->side_fork, st)) != cudaSuccess ||
                    (e = cudaStreamWaitEvent(p->side, p->side_fork, 0)) != cudaSuccess ||
                    (e = launch_blocks_sums<T>(p, a, blk, p->side)) != cudaSuccess ||
                    (e = cudaEventRecord(p->side_join, p->side)) != cudaSuccess))
-        return cuda_fail(e, "block convolution launch");
+        return leave(e, "block convolution launch");
     e = p->merged ? launch_pass_n<T>(zero_rim_fwd_pass(p), p->logN, a, 0, st,
                                      nullptr, p->tc)
                   : launch_pass_n<T>(general_fwd_pass(p), p->logN, a, (int)p->items.size(), st, nullptr, p->tc);
     if (e != cudaSuccess)
-        return cuda_fail(e, "row_fwd launch");
+        return leave(e, "row_fwd launch");
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
     e = launch_col<T>(p, a, st);
     if (e != cudaSuccess)
-        return cuda_fail(e, "col launch");
+        return leave(e, "col launch");
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
     if ((e = launch_row_inv<T>(p->logN, L, p->fo.R, a, st, p->tc, p->sched.row_inv0, p->sched.inv_radix,
                                p->tmap_inv2, p->blk)) !=
         cudaSuccess)
-        return cuda_fail(e, "row_inv launch");
+        return leave(e, "row_inv launch");
     if ((ms = mark(p, st)) != SGF_OK)
         return ms;
     if (p->blk) {
         e = beside ? cudaStreamWaitEvent(st, p->side_join, 0) : launch_blocks_sums<T>(p, a, blk, st);
         if (e != cudaSuccess || (e = launch_blocks_add<T>(a, blk, st)) != cudaSuccess)
-            return cuda_fail(e, "block convolution launch");
+            return leave(e, "block convolution launch");
     }
     return mark(p, st);
 }

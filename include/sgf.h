@@ -122,8 +122,8 @@ typedef struct sgf_plan sgf_plan;
 /* Per-plan counts, for reporting.  All sizes in bytes. */
 typedef struct {
     int32_t n, levels, precision;  /* levels: patches of a forest plan */
-    int32_t forward_slabs;      /* row-transformed source sets per solve (1 per level + Case-2 phases) */
-    int32_t outputs;            /* column-pass outputs per solve (1 per level + Case-3 phases) */
+    int32_t forward_slabs;      /* row-transformed source sets per solve: 1 per patch + the m^2 phases (blocks) of its pairs */
+    int32_t outputs;            /* column-pass outputs per solve: 1 per patch + the m^2 blocks (phases) of its pairs */
     int32_t spectra_sets;       /* kernel-spectrum sets (Case 1 shared; one per Case-2/3 phase) */
     int32_t launches_per_solve; /* kernels one sgf_solve launches */
     size_t workspace_bytes;     /* device workspace owned by this plan */
@@ -224,7 +224,8 @@ sgf_status sgf_plan_check(sgf_plan *plan);
 sgf_status sgf_plan_share(const sgf_plan *src, sgf_plan **out);
 
 /* As sgf_plan_share, with the new plan's precision: src's own, or SGF_FP32 and
- * SGF_BF16X for each other (both keep FP32 spectra).  Errors: SGF_EINVAL for
+ * SGF_BF16X for each other (both keep FP32 spectra).  Cross-level pairs run as
+ * src's spectra are stored: where src keeps block spectra, in FP32.  Errors: SGF_EINVAL for
  * another precision, SGF_EUNSUPPORTED where SGF_BF16X does not apply (n = 4096
  * with levels > 1), SGF_ENOMEM, SGF_ECUDA. */
 sgf_status sgf_plan_share_ex(const sgf_plan *src, sgf_precision precision, sgf_plan **out);

@@ -446,7 +446,8 @@ sgf_status sgf_solve_noalloc(sgf_plan *plan, const void *const *sigma, void *con
  *     its three fields from one staging of its sigma rows), each staging its
  *     next item's rows behind the current transforms.
  * A new plan starts from {0, 0, 0}, or from the schedule the autotuner recorded for
- * its key (device, n, precision, zero-rim, levels > 1); sgf_plan_share copies it. */
+ * its key (device, n, precision, zero-rim, levels > 1, potential, cross-level pairs as block
+ * convolutions); sgf_plan_share copies it. */
 typedef struct {
     int32_t col_pass;
     int32_t row_inv0;

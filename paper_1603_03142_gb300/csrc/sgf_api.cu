@@ -2544,8 +2544,10 @@ std::string tune_key(const sgf_plan *p)
         if (*c == ' ')
             *c = '_';
     char buf[160];
-    snprintf(buf, sizeof buf, "%s/n%d/p%d/zr%d/ml%d%s", dev, p->N, (int)p->prec, p->merged ? 1 : 0, p->L > 1 ? 1 : 0,
-             p->pot ? "/phi" : "");
+    // plans with block convolutions run other column and inverse row kernels (quarter spectra alone,
+    // no Case-3 outputs) than the whole-grid ones of the same size
+    snprintf(buf, sizeof buf, "%s/n%d/p%d/zr%d/ml%d%s%s", dev, p->N, (int)p->prec, p->merged ? 1 : 0, p->L > 1 ? 1 : 0,
+             p->pot ? "/phi" : "", p->blk ? "/blk" : "");
     return buf;
 }
 

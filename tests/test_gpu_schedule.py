@@ -225,6 +225,33 @@ print(json.dumps(sgf.Plan(W.Nest(n=1024), "fp32", zero_rim=True).schedule()))
     assert json.loads(out2.stdout.strip().splitlines()[-1]) == ch
 
 
+def test_block_and_whole_grid_plans_have_records_of_their_own(lib, tmp_path):
+    """Plans of one size and precision run other column and inverse row kernels with block
+    convolutions than with the whole-grid passes (here: over a spectra budget): tuning
+    either leaves the other's record as it was."""
+    table = tmp_path / "tune.txt"
+    code = r"""
+import sys, json
+sys.path.insert(0, %r)
+from paper_1603_03142_gb300 import sgf, workloads as W
+nest = W.centred_nest(256, 2)
+block = sgf.Plan(nest, "fp32")
+whole = sgf.Plan(nest, "fp32", spectra_budget=block.stats()["spectra_bytes"] // 2)
+assert whole.stats()["spectra_sets_streamed"] > 0
+block.autotune(reps=1)
+first = open(%r).read().split("\n")
+whole.autotune(reps=1)
+print(json.dumps({"first": first, "both": open(%r).read().split("\n")}))
+""" % (str(ROOT), str(table), str(table))
+    env = dict(os.environ, SGF_AUTOTUNE_CACHE=str(table))
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0, out.stderr
+    import json
+    d = json.loads(out.stdout.strip().splitlines()[-1])
+    first, both = ([ln for ln in d[k] if ln] for k in ("first", "both"))
+    assert len(first) == 1 and len(both) == 2 and first[0] in both
+
+
 @pytest.mark.parametrize("case", ["zero_rim_4096", "general_1024", "nest_512", "potential_1024"])
 def test_tma_gather_matches_lane_gather(lib, case):
     """row_inv0 = 3 (k_row_inv1t), 4 (k_row_inv1x) and 5 (k_row_inv2x) against

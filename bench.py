@@ -236,22 +236,31 @@ def time_forest(args, world, dev, stream):
 
 
 def nest_pair_bytes(nests, w: int = 4):
-    """Algorithmic HBM bytes of one solve of each nest (one patch per level, force
-    plans, w bytes per real), split by pair of levels: the same accounting as the
-    library's plan statistics (every intermediate written and read once, every
-    kernel spectrum read once per use, padding not counted).  Case 1 carries the
-    level's own forward slab and main output; a Case-2 pair (finer source, m =
-    2^d) its m^2 phase slabs of n/m rows and m^2 phase spectra; a Case-3 pair
-    (coarser source) its m^2 phase outputs of n/m rows and m^2 phase spectra:
-    bytes grow with m for the intermediates and m^2 for the spectra."""
+    """Algorithmic HBM bytes of one solve of each nest (one patch per level, FP32
+    force plans, n a power of two), split by pair of levels: the accounting of the
+    library's plan statistics (every intermediate written and read once, padding
+    not counted, kernel spectra as they are read).  Case 1 carries the level's own
+    forward slab and main output.  A Case-2 pair (finer source, m = 2^d) and a
+    Case-3 pair (coarser source) run as block convolutions from n = 256 on (blocks
+    of B = n/m >= 16 cells): m^2 units of (B + 1) 2B frequencies in and out, each
+    passing memory three times over, m^4 kernel blocks, and the forces read and
+    written once more; elsewhere as m^2 phases of n/m rows on the whole grid with
+    m^2 full spectra.  The kernel blocks of a pair centred along an axis are read
+    by half there, and one read serves up to four right-hand sides (two with mirror
+    images): the level pairs of one relative position and, in a batch of several
+    nests of one shape (nests with equal key()), the nests."""
     C = 2 * w
-    out = {}
+    out, readers = {}, {}
 
     def add(key, b):
         out[key] = out.get(key, 0) + b
     for nest in nests:
         n, L = int(nest.n), int(nest.levels)
         n1 = n + 1
+        blocks = L > 1 and n >= 256 and (n >> (L - 1)) >= 16
+        org = [(0, 0)]
+        for l in range(1, L):
+            org.append(tuple(2 * (org[-1][a] + nest.off[l][a]) for a in range(2)))
         add("sigma_in_forces_out", 3 * L * n * n * w)
         if L > 1:  # restriction of every covered level: its input, its copy, the children of its covered cells
             add("restriction", (L - 1) * (2 * n * n * w + 4 * (n // 2) ** 2 * w))
@@ -262,11 +271,25 @@ def nest_pair_bytes(nests, w: int = 4):
                     continue
                 d = abs(s - t)
                 m = 1 << d
+                case = 2 if s > t else 3  # finer source, coarser source
+                if blocks:
+                    B = n // m
+                    F = (B + 1) * 2 * B
+                    add(f"case{case}_d{d}", (3 + 2) * 3 * m * m * F * C + 2 * 2 * n * n * w)
+                    at = tuple(org[max(s, t)][a] - m * org[min(s, t)][a] for a in range(2))
+                    key = (nest.key(), case, d, at)
+                    readers[key] = readers.get(key, 0) + 1
+                    continue
                 spec = m * m * 6 * n1 * 2 * n * C
-                if s > t:  # Case 2: finer source, m^2 phase slabs of n/m rows
+                if case == 2:  # m^2 phase slabs of n/m rows
                     add(f"case2_d{d}", spec + 2 * 3 * n1 * n * C * m)
-                else:      # Case 3: coarser source, m^2 phase outputs of n/m rows
+                else:          # m^2 phase outputs of n/m rows
                     add(f"case3_d{d}", spec + 2 * 2 * n1 * n * C * m)
+    for (shape, case, d, at), count in readers.items():
+        n, m = int(shape[0]), 1 << d
+        mirrored = sum(a == n // 2 * (m - 1) for a in at)
+        blk = 6 * (n // m + 1) * 2 * (n // m) * C
+        add(f"case{case}_d{d}", -(-count // (2 if mirrored else 4)) * (m ** 4 >> mirrored) * blk)
     tot = sum(out.values())
     return {"bytes": out, "total": tot, "share": {k: v / tot for k, v in out.items()}}
 
@@ -671,8 +694,8 @@ def run_batched(args, world, rank, local):
         ms = float(t.item())
     cells = sum(probs[k][0].levels * probs[k][0].n ** 2 for k in range(len(probs)))
     spectra_gib = sum(p.stats()["spectra_bytes"] for p in base.values()) / 2**30
-    algo = sum(plans[i].stats()["algorithmic_bytes"] for i in range(len(plans)))
     pairs = nest_pair_bytes([probs[k][0] for k in mine])
+    algo = pairs["total"]  # the plans' own figures count a shared read of kernel spectra once per plan
     batch.close()
     for p in plans:
         p.close()

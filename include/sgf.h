@@ -128,8 +128,10 @@ typedef struct {
     int32_t launches_per_solve; /* kernels one sgf_solve launches */
     size_t workspace_bytes;     /* device workspace owned by this plan */
     size_t spectra_bytes;       /* device kernel spectra (shared between plans made by sgf_plan_share) */
-    size_t algorithmic_bytes;   /* HBM bytes one solve must move: inputs, outputs, spectra and
-                                   the two transposed intermediates, each read or written once */
+    size_t algorithmic_bytes;   /* HBM bytes one solve must move: inputs, outputs and the transposed
+                                   intermediates of every pass, and the kernel spectra it reads (of a
+                                   pair that is mirror-symmetric along an axis half, along both a
+                                   quarter; once for the pairs whose products share a read) */
     double plan_ms;             /* wall time spent building the spectra */
     int32_t spectra_sets_streamed; /* sets regenerated at every solve (spectra budget), else 0 */
     int32_t spectra_waves;      /* window refills per solve (spectra budget), else 0 */

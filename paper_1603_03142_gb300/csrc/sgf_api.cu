@@ -607,6 +607,10 @@ int blk_tw_offset(int logB)
 // components, R right-hand sides) have to stay in registers.
 int mac_qg(int qg, int rhs, int sym) { return std::min(qg, sym ? 1 : rhs == 1 ? 4 : rhs == 2 ? 2 : 1); }
 
+// Target units a work item's products run over: with mirror images summed too, half of them per
+// mirrored axis.
+int mac_units(const MacItem &it) { return it.m2 >> ((it.sym & kMirrorX ? 1 : 0) + (it.sym & kMirrorY ? 1 : 0)); }
+
 // Work items of the products: targets whose terms read the same kernel spectra
 // share them, up to four right-hand sides an item, two where mirror images are summed
 // too (the accumulators of more do not fit in registers).  QG targets per warp
@@ -661,26 +665,33 @@ void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &
             items.push_back(it);
         }
     }
-    auto units = [](const MacItem &it) {  // target units the warps run over
-        return it.m2 >> ((it.sym & kMirrorX ? 1 : 0) + (it.sym & kMirrorY ? 1 : 0));
-    };
     int qg = 4;
     for (; qg > 1; qg >>= 1) {
         long long warps = 0;
         for (const auto &it : items)
-            warps += (long long)it.tiles * std::max(1, units(it) / mac_qg(qg, it.rhs, it.sym));
+            warps += (long long)it.tiles * std::max(1, mac_units(it) / mac_qg(qg, it.rhs, it.sym));
         if (warps >= 16 * 152)
             break;
     }
     for (auto &it : items) {
-        it.qg = std::min(units(it), mac_qg(qg, it.rhs, it.sym));
-        it.nqg = units(it) / it.qg;
+        it.qg = std::min(mac_units(it), mac_qg(qg, it.rhs, it.sym));
+        it.nqg = mac_units(it) / it.qg;
         int &blk = it.sym ? launch->sym_blocks : launch->blocks;
         (it.sym ? launch->sym_items : launch->items)++;
         it.blk_begin = blk;
         const long long warps = (long long)it.tiles * it.nqg;
         blk += (int)((warps + kBlkThreads / 32 - 1) / (kBlkThreads / 32));
     }
+}
+
+// Bytes of kernel spectra the products read: every block of those units once per item, whatever
+// number of right-hand sides it serves.
+size_t mac_bytes(const std::vector<MacItem> &items, int ncomp, size_t Cb)
+{
+    size_t b = 0;
+    for (const auto &it : items)
+        b += (size_t)it.term_count * it.m2 * mac_units(it) * 3 * ncomp * it.F * Cb;
+    return b;
 }
 
 // The stages, sources, targets and products of a plan's cross-level pairs; off:
@@ -1065,15 +1076,13 @@ void build_lists(sgf_plan *p)
             ab += 2 * (size_t)N * N * T + 4 * cov * T;
         }
     // block convolutions: every source and target field written and read twice (rows, columns), the
-    // kernel spectra of every pair read once, the forces read and written where a pair adds to them
+    // forces read and written where a pair adds to them, the kernel spectra as the products read them
     for (const auto &sg : p->stages) {
         const size_t fld = (size_t)sg.m * sg.m * blk_freqs(sg.logB) * Cb;
         ab += 3 * fld * 3 * sg.src_count + ncomp * fld * 3 * (sg.tgt_count[0] + sg.tgt_count[1]) +
               2 * ncomp * (size_t)N * N * T * (sg.tgt_count[0] + sg.tgt_count[1]);
     }
-    for (const auto &bt : p->btargets)
-        ab += bt.terms.size() * (size_t)bt.m2 * bt.m2 * 3 * ncomp * bt.F * Cb;
-    p->algorithmic_bytes = ab;
+    p->algorithmic_bytes = ab + mac_bytes(p->mitems, (int)ncomp, Cb);
 }
 
 // Stored bytes of one spectra set (256-byte aligned).

@@ -110,3 +110,19 @@ def test_profile_commands_use_flags_bench_accepts():
     assert flags, "no bench.py command found under profiles/"
     missing = sorted(fl for fl in flags if fl not in helptext)
     assert not missing, missing
+
+
+def test_nest_pair_bytes_count_spectra_as_they_are_read(bench):
+    """Kernel blocks of a pair centred along an axis are read by half there, and one
+    read serves four right-hand sides (two with mirror images)."""
+    from paper_1603_03142_gb300 import workloads as W
+    n, m, B = 512, 2, 256
+    sets = m ** 4 * 6 * (B + 1) * 2 * B * 8
+    fields = 5 * 3 * m * m * (B + 1) * 2 * B * 8 + 2 * 2 * n * n * 4
+
+    def case2(*nests):
+        return bench.nest_pair_bytes(list(nests))["bytes"]["case2_d1"] - len(nests) * fields
+    off, on_y, centred = (W.Nest(n=n, levels=2, off=[(0, 0), o]) for o in ((100, 7), (100, 128), (128, 128)))
+    assert case2(off) == sets and case2(on_y) == sets // 2 and case2(centred) == sets // 4
+    assert case2(off, off, off, off) == sets and case2(*[off] * 5) == 2 * sets and case2(off, on_y) == 3 * sets // 2
+    assert case2(centred, centred) == sets // 4 and case2(*[centred] * 3) == sets // 2

@@ -159,3 +159,14 @@ def test_bf16x_depths_and_shared_spectra(lib):
             for l in range(levels):
                 scale = max(np.abs(ref[0][l]).max(), np.abs(ref[1][l]).max())
                 assert max(np.abs(got[c][l] - ref[c][l]).max() for c in range(2)) <= tol("bf16x", n) * scale
+
+
+@pytest.mark.parametrize("n,levels,centre", [(256, 3, (0.0, 0.0)), (256, 4, (0.3, 0.0)), (256, 3, (0.3, -0.2)),
+                                             (512, 2, (0.0, 0.0)), (128, 3, (0.0, 0.0)), (256, 1, (0.0, 0.0))])
+def test_algorithmic_bytes_follow_the_reads(lib, n, levels, centre):
+    """The plan's byte count is that of bench.py's split by pair of levels: the spectra as the
+    products read them (halves and quarters of mirror-symmetric pairs, shared reads once)."""
+    from bench import nest_pair_bytes
+    nest = W.centred_nest(n, levels, centre=centre) if levels > 1 else W.Nest(n=n)
+    plan = lib.Plan(nest, "fp32")
+    assert plan.stats()["algorithmic_bytes"] == nest_pair_bytes([nest])["total"]

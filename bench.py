@@ -186,6 +186,26 @@ def run_reference(args, world, rank):
     print(json.dumps(line), flush=True)
 
 
+def time_solves(plan, step, steps, stream):
+    """ms per solve (CUDA events around `steps` solves, as a caller runs them), then the
+    plan's per-kernel times from as many profiled solves: those run every pass one after
+    the other, also where a small nest's block convolutions run beside its own passes."""
+    import torch
+    ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    ev0.record(stream)
+    for k in range(steps):
+        step(k)
+    ev1.record(stream)
+    torch.cuda.synchronize()
+    plan.profile(True)
+    for k in range(steps):
+        step(k)
+    torch.cuda.synchronize()
+    plan.profile(False)
+    return ev0.elapsed_time(ev1) / steps, plan.profile_read()
+
+
 def time_forest(args, world, dev, stream):
     """Example 3's geometry (Sec. 3: two disks, six level-0 tiles and two level-1
     patches of forest_n^2 cells each, the paper's N = 2 forest_n), FP32: ms per
@@ -209,17 +229,7 @@ def time_forest(args, world, dev, stream):
                         [a.data_ptr() for a in fy[k % sets]], stream)
     for k in range(args.warmup):
         step(k)
-    torch.cuda.synchronize()
-    plan.profile(True)
-    ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    ev0.record(stream)
-    for k in range(args.steps):
-        step(k)
-    ev1.record(stream)
-    torch.cuda.synchronize()
-    plan.profile(False)
-    ms = ev0.elapsed_time(ev1) / args.steps
-    prof = plan.profile_read()
+    ms, prof = time_solves(plan, step, args.steps, stream)
     st = plan.stats()
     cells = sum(a.numel() for a in sig0)
     out = {"workload": f"two-disk forest (Example 3): 6 level-0 + 2 level-1 patches of {args.forest_n}^2",
@@ -620,18 +630,8 @@ def run_nest_solves(args, world, rank, local):
                         [a.data_ptr() for a in fy[q]], stream)
     for k in range(args.warmup):
         step(k)
-    torch.cuda.synchronize()
-    plan.profile(True)
-    ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    ev0.record(stream)
-    for k in range(args.steps):
-        step(k)
-    ev1.record(stream)
-    torch.cuda.synchronize()
-    plan.profile(False)
+    ms, prof = time_solves(plan, step, args.steps, stream)
     plan.check()
-    prof = plan.profile_read()
-    ms = ev0.elapsed_time(ev1) / args.steps
     if rank == 0:
         print(json.dumps({"mode": "solve-only", "n": args.n, "levels": args.nest_levels, "ms_per_step": ms,
                           "cells_per_s": args.nest_levels * args.n * args.n / (ms / 1e3),

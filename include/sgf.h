@@ -330,7 +330,8 @@ sgf_status sgf_batch_destroy(sgf_batch *batch);
 
 /* Per-kernel device times of this plan's solves, for measurement (no paper
  * counterpart).  Kernel k: 0 restriction, 1 forward row pass, 2 column pass
- * (with the spectral multiply-accumulate), 3 inverse row pass. */
+ * (with the spectral multiply-accumulate, and every pass of the cross-level
+ * pairs that run as block convolutions), 3 inverse row pass. */
 typedef struct {
     int32_t solves;       /* solves recorded since the last read */
     int32_t launches[4];  /* launches per kernel */
@@ -339,7 +340,10 @@ typedef struct {
 
 /* enable != 0: every later sgf_solve on this plan records CUDA events around
  * its kernel launches on the solve's stream (events are created on first
- * use); enable == 0 stops recording. */
+ * use); enable == 0 stops recording.  Recorded solves run their passes one
+ * after the other, also where a small plan's cross-level pairs otherwise run
+ * beside its patches' own passes (n <= 512): their total is then above an
+ * unrecorded solve's. */
 sgf_status sgf_plan_profile(sgf_plan *plan, int32_t enable);
 
 /* Waits for the recorded solves, returns their summed times and clears them. */

@@ -126,3 +126,38 @@ def test_nest_pair_bytes_count_spectra_as_they_are_read(bench):
     assert case2(off) == sets and case2(on_y) == sets // 2 and case2(centred) == sets // 4
     assert case2(off, off, off, off) == sets and case2(*[off] * 5) == 2 * sets and case2(off, on_y) == 3 * sets // 2
     assert case2(centred, centred) == sets // 4 and case2(*[centred] * 3) == sets // 2
+
+
+def test_solves_are_timed_with_profiling_off(bench, monkeypatch):
+    """A profiled solve runs its passes one after the other: the solves between the timing
+    events are unprofiled ones, the per-kernel times come from as many profiled ones after."""
+    import torch
+    log = []
+
+    class Event:
+        def __init__(self, enable_timing=False):
+            pass
+
+        def record(self, stream=None):
+            log.append("event")
+
+        def elapsed_time(self, other):
+            return 6.0
+
+    class Plan:
+        on = False
+
+        def profile(self, enable):
+            self.on = enable
+
+        def profile_read(self):
+            return {"solves": log.count("profiled")}
+    plan = Plan()
+    monkeypatch.setattr(torch.cuda, "Event", Event)
+    monkeypatch.setattr(torch.cuda, "synchronize", lambda: None)
+    ms, prof = bench.time_solves(plan, lambda k: log.append("profiled" if plan.on else "plain"), 3, None)
+    assert log == ["event"] + ["plain"] * 3 + ["event"] + ["profiled"] * 3
+    assert ms == 2.0 and prof["solves"] == 3 and not plan.on
+    for name in ("time_forest", "run_nest_solves"):
+        code = getattr(bench, name).__code__
+        assert "time_solves" in code.co_names and "profile" not in code.co_names

@@ -156,8 +156,8 @@ __device__ __forceinline__ float2 ld_stream(const float2 *p)
     return v;
 }
 
-template <typename T, int NC, int SYM, int QG, int R>
-__device__ __forceinline__ void mac_sym_body(const MacArgs<T> &m, const MacItem &it, int tile, int q0, int lane)
+template <typename T, int NC, int SYM, int R>
+__device__ __forceinline__ void mac_sym_body(const MacArgs<T> &m, const MacItem &it, int tile, int unit, int lane)
 {
     using C = typename Cx<T>::C;
     constexpr bool SX = (SYM & kMirrorX) != 0, SY = (SYM & kMirrorY) != 0;
@@ -177,30 +177,25 @@ __device__ __forceinline__ void mac_sym_body(const MacArgs<T> &m, const MacItem 
         const bool mx = SX && (e & 1), my = SY && (SX ? (e & 2) != 0 : (e & 1) != 0);
         return ((my ? mm - 1 - y : y) << it.logm) + (mx ? mm - 1 - x : x);
     };
-    int q[QG];
     const int lq = SX ? it.logm - 1 : it.logm;  // base units: the lower half in the mirrored axes
+    const int q = ((unit >> lq) << it.logm) + (unit & ((1 << lq) - 1));
+    C sa[IM][NC][R], sb[IM][NC][R];
 #pragma unroll
-    for (int g = 0; g < QG; ++g)
-        q[g] = (((q0 + g) >> lq) << it.logm) + ((q0 + g) & ((1 << lq) - 1));
-    C sa[QG][IM][NC][R], sb[QG][IM][NC][R];
+    for (int e = 0; e < IM; ++e)
 #pragma unroll
-    for (int g = 0; g < QG; ++g)
+        for (int c = 0; c < NC; ++c)
 #pragma unroll
-        for (int e = 0; e < IM; ++e)
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-                    sa[g][e][c][r] = sb[g][e][c][r] = hmk<C>(T(0), T(0));
+            for (int r = 0; r < R; ++r)
+                sa[e][c][r] = sb[e][c][r] = hmk<C>(T(0), T(0));
     for (int tm = 0; tm < it.term_count; ++tm) {
         const MacTerm te = m.terms[it.term_begin + tm];
         const C *xb0[R];
 #pragma unroll
         for (int r = 0; r < R; ++r)
             xb0[r] = m.x + m.xo[te.x_begin + r];
-#pragma unroll (R == 1 && QG == 1 ? 2 : 1)
+#pragma unroll (R == 1 ? 2 : 1)
         for (int p = 0; p < it.m2; ++p) {
-            const C *kp = m.spec + te.k_off + (size_t)p * te.sp;
+            const C *kp = m.spec + te.k_off + (size_t)p * te.sp + (size_t)q * te.sq;
 #pragma unroll
             for (int f = 0; f < 3; ++f) {
                 C xa[IM][R], xb[IM][R];
@@ -213,23 +208,21 @@ __device__ __forceinline__ void mac_sym_body(const MacArgs<T> &m, const MacItem 
                         xb[e][r] = __ldg(x + fb);
                     }
 #pragma unroll
-                for (int g = 0; g < QG; ++g)
+                for (int c = 0; c < NC; ++c) {
+                    const C *kk = kp + (size_t)(c * 3 + f) * F;
+                    const C ka = ld_stream(kk + fa), kb = ld_stream(kk + fb);
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        const C *kk = kp + (size_t)q[g] * te.sq + (size_t)(c * 3 + f) * F;
-                        const C ka = ld_stream(kk + fa), kb = ld_stream(kk + fb);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            mac_pair<NC, false, false>(sa[g][0][c][r], sb[g][0][c][r], ka, kb, xa[0][r], xb[0][r], c, f);
-                            if constexpr (SX)
-                                mac_pair<NC, true, false>(sa[g][1][c][r], sb[g][1][c][r], ka, kb, xa[1][r], xb[1][r], c, f);
-                            if constexpr (SY)
-                                mac_pair<NC, false, true>(sa[g][IM / 2][c][r], sb[g][IM / 2][c][r], ka, kb, xa[IM / 2][r],
-                                                          xb[IM / 2][r], c, f);
-                            if constexpr (SX && SY)
-                                mac_pair<NC, true, true>(sa[g][3][c][r], sb[g][3][c][r], ka, kb, xa[3][r], xb[3][r], c, f);
-                        }
+                    for (int r = 0; r < R; ++r) {
+                        mac_pair<NC, false, false>(sa[0][c][r], sb[0][c][r], ka, kb, xa[0][r], xb[0][r], c, f);
+                        if constexpr (SX)
+                            mac_pair<NC, true, false>(sa[1][c][r], sb[1][c][r], ka, kb, xa[1][r], xb[1][r], c, f);
+                        if constexpr (SY)
+                            mac_pair<NC, false, true>(sa[IM / 2][c][r], sb[IM / 2][c][r], ka, kb, xa[IM / 2][r],
+                                                      xb[IM / 2][r], c, f);
+                        if constexpr (SX && SY)
+                            mac_pair<NC, true, true>(sa[3][c][r], sb[3][c][r], ka, kb, xa[3][r], xb[3][r], c, f);
                     }
+                }
             }
         }
     }
@@ -237,15 +230,13 @@ __device__ __forceinline__ void mac_sym_body(const MacArgs<T> &m, const MacItem 
     for (int r = 0; r < R; ++r) {
         C *dst = m.acc + m.ao[it.a_begin + r];
 #pragma unroll
-        for (int g = 0; g < QG; ++g)
+        for (int e = 0; e < IM; ++e)
 #pragma unroll
-            for (int e = 0; e < IM; ++e)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    C *o = dst + ((size_t)mirror(q[g], e) * NC + c) * F;
-                    o[fa] = sa[g][e][c][r];
-                    o[fb] = sb[g][e][c][r];  // ky = 0 and the Nyquist bin: the same value again
-                }
+            for (int c = 0; c < NC; ++c) {
+                C *o = dst + ((size_t)mirror(q, e) * NC + c) * F;
+                o[fa] = sa[e][c][r];
+                o[fb] = sb[e][c][r];  // ky = 0 and the Nyquist bin: the same value again
+            }
     }
 }
 
@@ -303,33 +294,22 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_blk_mac_sym(MacArgs<T> m)
     if (!mac_locate(m, it, tile, q0))
         return;
     const int lane = threadIdx.x & 31;
-    auto run = [&](auto sym, auto qg, auto rhs) {
-        mac_sym_body<T, NC, decltype(sym)::value, decltype(qg)::value, decltype(rhs)::value>(m, it, tile, q0, lane);
-    };
-    constexpr std::integral_constant<int, 1> one{};
-    constexpr std::integral_constant<int, 2> two{};
-    constexpr std::integral_constant<int, 3> both{};
-    if (it.sym == both) {
+    // one unit and its images a warp (mac_qg), one or two right-hand sides
+    if (it.sym == (kMirrorX | kMirrorY)) {
         if (it.rhs == 2)
-            run(both, one, two);
-        else if (it.qg == 2)
-            run(both, two, one);
+            mac_sym_body<T, NC, kMirrorX | kMirrorY, 2>(m, it, tile, q0, lane);
         else
-            run(both, one, one);
+            mac_sym_body<T, NC, kMirrorX | kMirrorY, 1>(m, it, tile, q0, lane);
     } else if (it.sym == kMirrorX) {
         if (it.rhs == 2)
-            run(one, one, two);
-        else if (it.qg == 2)
-            run(one, two, one);
+            mac_sym_body<T, NC, kMirrorX, 2>(m, it, tile, q0, lane);
         else
-            run(one, one, one);
+            mac_sym_body<T, NC, kMirrorX, 1>(m, it, tile, q0, lane);
     } else {
         if (it.rhs == 2)
-            run(two, one, two);
-        else if (it.qg == 2)
-            run(two, two, one);
+            mac_sym_body<T, NC, kMirrorY, 2>(m, it, tile, q0, lane);
         else
-            run(two, one, one);
+            mac_sym_body<T, NC, kMirrorY, 1>(m, it, tile, q0, lane);
     }
 }
 

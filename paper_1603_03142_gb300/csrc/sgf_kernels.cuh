@@ -2619,9 +2619,9 @@ __global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS, 1) k_col_mw(Sol
 #pragma unroll
                 for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
-                    if (b == 1 && u < 8)
+                    if (b == 1 && u < K::V / 2)
                         fold[n] = hmulc(acc[0][u], twist_v<C, K::V>(tw, tl, N, j, u));
-                    else if (b == 0 && u >= 8)
+                    else if (b == 0 && u >= K::V / 2)
                         fold[n] = acc[0][u];
                 }
             }
@@ -2630,9 +2630,9 @@ __global__ void __launch_bounds__(KShape<LOGN, TC>::ROW_THREADS, 1) k_col_mw(Sol
 #pragma unroll
                 for (int u = 0; u < K::V; ++u) {
                     const int n = j + u * Q;
-                    if (b == 0 && u < 8)
+                    if (b == 0 && u < K::V / 2)
                         dst[bwd_index(N, N, 0, kx, n)] = hadd(acc[0][u], fold[n]);
-                    else if (b == 1 && u >= 8)
+                    else if (b == 1 && u >= K::V / 2)
                         dst[bwd_index(N, N, 0, kx, n)] = hadd(fold[n], hmulc(acc[0][u], twist_v<C, K::V>(tw, tl, N, j, u)));
                 }
             }

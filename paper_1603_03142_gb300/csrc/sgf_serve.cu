@@ -342,9 +342,9 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
     Pending p;
     p.r = *r;
     // FP32 and SGF_BF16X requests of a shape share its spectra: from three levels on, where
-    // SGF_BF16X plans keep the whole-grid passes, every request of the shape does (the
-    // per-shape cap goes by sgf_plan_estimate all the same)
-    p.whole_grid = r->desc.levels >= 3;
+    // SGF_BF16X plans keep the whole-grid passes, every such request of the shape does (the
+    // per-shape cap goes by sgf_plan_estimate all the same); SGF_FP64 ones share with none
+    p.whole_grid = r->desc.levels >= 3 && r->precision != SGF_FP64;
     size_t pub_ws = 0, pub_spectra = 0, pub_build = 0;
     sgf_status rc = sgf_plan_estimate(&r->desc, r->precision, r->plan_flags, &pub_ws, &pub_spectra, &pub_build);
     if (rc == SGF_OK)

@@ -203,3 +203,16 @@ def test_max_shape_bytes_rejects_large_shapes():
     assert [d["id"] for d in _drain(srv, 1)] == [1]
     assert srv.stats()["rejected"] == 1
     srv.close()
+
+
+def test_fp64_requests_run_as_plans_do():
+    """SGF_FP64 spectra are shared with no other precision: such a request takes the passes, and
+    the memory, of the plan sgf_plan_create_ex makes, at any depth."""
+    nest = W.centred_nest(256, 4, centre=(0.3, 0.1))
+    e = sgf.estimate(nest, "fp64")
+    srv = sgf.Server(hbm_budget=64 << 30, max_inflight=1, simulate_gbs=100.0)
+    arrays = [[np.ones((256, 256)) for _ in range(4)] for _ in range(3)]
+    assert srv.submit(0, nest, "fp64", *arrays) == 0
+    _drain(srv, 1)
+    assert srv.stats()["bytes_used"] == e["workspace_bytes"] + e["spectra_bytes"] + 3 * 4 * 256 * 256 * 8
+    srv.close()

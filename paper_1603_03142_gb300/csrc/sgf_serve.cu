@@ -372,16 +372,21 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
             return rc;
     }
     if (sv->cfg.max_shape_bytes && shape_bytes > sv->cfg.max_shape_bytes &&
-        (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0 && p.build < sv->cfg.max_shape_bytes) {
-        // served by plans over a spectra budget: resident sets and a window within the budget,
-        // the generator's workspace kept by every slot's plan
+        (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0) {
+        // served by plans over a spectra budget: resident sets and a window within the budget, the
+        // generator's workspace kept by every slot's plan; such plans run the whole-grid passes
+        size_t ws = 0, spectra = 0, build = 0;
+        rc = nest_plan_estimate(&r->desc, r->precision, 0, true, &ws, &spectra, &build);
+        if (rc != SGF_OK)
+            return rc;
         const size_t esz = r->precision == SGF_FP64 ? 8 : 4;
         const size_t one_set = 6 * (size_t)(r->desc.n + 1) * 2 * r->desc.n * 2 * esz;
-        const size_t budget = sv->cfg.max_shape_bytes - p.build;
-        if (budget >= one_set) {
-            p.stream_budget = budget;
-            p.ws += p.build + budget;  // generator workspace and (at most) the window, per slot
-            p.spectra = budget;        // the resident sets, at most the budget
+        if (build < sv->cfg.max_shape_bytes && sv->cfg.max_shape_bytes - build >= one_set) {
+            p.whole_grid = true;
+            p.stream_budget = sv->cfg.max_shape_bytes - build;
+            p.ws = ws + build + p.stream_budget;  // generator workspace and (at most) the window, per slot
+            p.spectra = p.stream_budget;          // the resident sets, at most the budget
+            p.build = build;
         }
     }
     const size_t worst = p.ws + p.io + p.spectra + p.build;

@@ -216,3 +216,18 @@ def test_fp64_requests_run_as_plans_do():
     _drain(srv, 1)
     assert srv.stats()["bytes_used"] == e["workspace_bytes"] + e["spectra_bytes"] + 3 * 4 * 256 * 256 * 8
     srv.close()
+
+
+def test_streamed_shapes_are_charged_as_whole_grid_plans():
+    """A shape over the cap runs over a spectra budget, on the whole-grid passes: it is admitted
+    wherever their workspace fits (512^2, two levels: 42 MB, with the block convolutions' fields 63 MB)."""
+    nest = W.centred_nest(512, 2, centre=(0.3, 0.1))
+    e = sgf.estimate(nest, "fp32")
+    cap = e["build_bytes"] + e["spectra_bytes"] // 2
+    io = 3 * 2 * 512 * 512 * 4
+    need = (42 << 20) + (1 << 20) + io + 2 * cap  # workspace, lists, buffers; sets and window; generator twice
+    assert need < e["workspace_bytes"] + io + 2 * cap
+    srv = sgf.Server(hbm_budget=need, max_inflight=1, simulate_gbs=100.0, max_shape_bytes=cap, stream_large=True)
+    assert srv.submit(0, nest, "fp32", _arrays(512, 2), _arrays(512, 2), _arrays(512, 2)) == 0
+    _drain(srv, 1)
+    srv.close()

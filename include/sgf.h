@@ -551,9 +551,9 @@ typedef struct {
     int32_t max_inflight;  /* requests on the device at once, >= 1 */
     uint32_t flags;        /* SGF_SERVER_* */
     double simulate_gbs;   /* SGF_SERVER_SIMULATE: modelled rate in GB/s (> 0) */
-    size_t max_shape_bytes; /* 0, or the largest spectra + generator memory of one shape: requests of
-                               larger shapes are rejected at submit (SGF_ENOMEM) instead of evicting
-                               every other resident shape */
+    size_t max_shape_bytes; /* 0, or the largest spectra + generator memory (sgf_plan_estimate) of one
+                               shape: requests of larger shapes are rejected at submit (SGF_ENOMEM)
+                               instead of evicting every other resident shape */
 } sgf_server_config;
 
 /* One force request.  sigma[l], fx[l], fy[l] (l < desc.levels) are HOST arrays

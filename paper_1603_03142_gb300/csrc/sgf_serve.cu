@@ -342,8 +342,9 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
     Pending p;
     p.r = *r;
     // FP32 and SGF_BF16X requests of a shape share its spectra: from three levels on, where
-    // SGF_BF16X plans keep the whole-grid passes, every such request of the shape does (the
-    // per-shape cap goes by sgf_plan_estimate all the same); SGF_FP64 ones share with none
+    // SGF_BF16X plans keep the whole-grid passes, every such request of the shape does;
+    // SGF_FP64 ones share with none.  The per-shape cap goes by sgf_plan_estimate, whose block
+    // spectra hold (m - 1)/(N + 1) more of every pair (256^2: 0.4 % of two levels, 4 % of five).
     p.whole_grid = r->desc.levels >= 3 && r->precision != SGF_FP64;
     size_t pub_ws = 0, pub_spectra = 0, pub_build = 0;
     sgf_status rc = sgf_plan_estimate(&r->desc, r->precision, r->plan_flags, &pub_ws, &pub_spectra, &pub_build);
@@ -351,7 +352,8 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
         rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, p.whole_grid, &p.ws, &p.spectra, &p.build);
     if (rc != SGF_OK)
         return rc;
-    const size_t shape_bytes = std::max(p.spectra + p.build, pub_spectra + pub_build);
+    size_t shape_bytes = std::max(p.spectra + p.build, pub_spectra + pub_build);
+    const size_t cap = sv->cfg.max_shape_bytes;
     if (r->plan_flags & SGF_PLAN_POTENTIAL)
         return fail(SGF_EUNSUPPORTED, "request %llu: the request loop solves forces, not SGF_PLAN_POTENTIAL",
                     (unsigned long long)r->id);
@@ -363,16 +365,15 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
     p.io = 3 * (size_t)L * align256(lvl);
     p.skey = spectra_key(*r);
     p.key = p.skey + "/p" + std::to_string((int)r->precision);
-    if (!p.whole_grid && p.ws + p.io + p.spectra + p.build > sv->cfg.hbm_budget) {
-        // the block convolutions' spectra are up to 2% larger than the whole-grid passes': a shape
-        // that fits only as those is served so
+    if (!p.whole_grid && (p.ws + p.io + p.spectra + p.build > sv->cfg.hbm_budget || (cap && shape_bytes > cap))) {
+        // block convolutions that do not fit: with the whole-grid passes' spectra the shape may
         p.whole_grid = true;
         rc = nest_plan_estimate(&r->desc, r->precision, r->plan_flags, true, &p.ws, &p.spectra, &p.build);
         if (rc != SGF_OK)
             return rc;
+        shape_bytes = p.spectra + p.build;
     }
-    if (sv->cfg.max_shape_bytes && shape_bytes > sv->cfg.max_shape_bytes &&
-        (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0) {
+    if (cap && shape_bytes > cap && (sv->cfg.flags & SGF_SERVER_STREAM) && r->plan_flags == 0) {
         // served by plans over a spectra budget: resident sets and a window within the budget, the
         // generator's workspace kept by every slot's plan; such plans run the whole-grid passes
         size_t ws = 0, spectra = 0, build = 0;
@@ -381,19 +382,19 @@ sgf_status sgf_server_submit(sgf_server *sv, const sgf_request *r)
             return rc;
         const size_t esz = r->precision == SGF_FP64 ? 8 : 4;
         const size_t one_set = 6 * (size_t)(r->desc.n + 1) * 2 * r->desc.n * 2 * esz;
-        if (build < sv->cfg.max_shape_bytes && sv->cfg.max_shape_bytes - build >= one_set) {
+        if (build < cap && cap - build >= one_set) {
             p.whole_grid = true;
-            p.stream_budget = sv->cfg.max_shape_bytes - build;
+            p.stream_budget = cap - build;
             p.ws = ws + build + p.stream_budget;  // generator workspace and (at most) the window, per slot
             p.spectra = p.stream_budget;          // the resident sets, at most the budget
             p.build = build;
         }
     }
     const size_t worst = p.ws + p.io + p.spectra + p.build;
-    if (sv->cfg.max_shape_bytes && !p.stream_budget && shape_bytes > sv->cfg.max_shape_bytes) {
+    if (cap && !p.stream_budget && shape_bytes > cap) {
         sv->st.rejected++;
         return fail(SGF_ENOMEM, "request %llu: its shape needs %zu bytes of spectra and generator memory, above "
-                    "max_shape_bytes %zu", (unsigned long long)r->id, shape_bytes, sv->cfg.max_shape_bytes);
+                    "max_shape_bytes %zu", (unsigned long long)r->id, shape_bytes, cap);
     }
     if (worst > sv->cfg.hbm_budget) {
         sv->st.rejected++;

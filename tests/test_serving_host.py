@@ -231,3 +231,25 @@ def test_streamed_shapes_are_charged_as_whole_grid_plans():
     assert srv.submit(0, nest, "fp32", _arrays(512, 2), _arrays(512, 2), _arrays(512, 2)) == 0
     _drain(srv, 1)
     srv.close()
+
+
+@pytest.mark.parametrize("prec,levels", [("fp32", 2), ("bf16x", 2), ("fp64", 2), ("fp64", 4)])
+def test_shapes_that_fit_as_whole_grid_plans_are_served(prec, levels):
+    """Block spectra hold m^4 blocks of (N/m + 1) 2N/m values a pair where the whole-grid passes hold m^2
+    sets of (N + 1) 2N: a shape whose blocks alone are over the cap is served by those passes."""
+    n, w = 256, 8 if prec == "fp64" else 4
+    nest = W.centred_nest(n, levels, centre=(0.3, 0.2))
+    e = sgf.estimate(nest, prec)
+    more = sum(2 * (levels - d) * 4 ** d * 6 * 2 * n * 2 * w * (2 ** d - 1) for d in range(1, levels))
+    whole = e["spectra_bytes"] - more + sgf.estimate(W.Nest(n=n), prec)["build_bytes"]
+    assert whole < e["spectra_bytes"] + e["build_bytes"]
+    srv = sgf.Server(hbm_budget=64 << 30, max_inflight=1, simulate_gbs=100.0, max_shape_bytes=whole)
+    dt = np.float64 if prec == "fp64" else np.float32
+    arrays = [[np.ones((n, n), dt) for _ in range(levels)] for _ in range(3)]
+    assert srv.submit(0, nest, prec, *arrays) == 0
+    _drain(srv, 1)
+    assert srv.stats()["bytes_used"] < e["workspace_bytes"] + e["spectra_bytes"] + 3 * levels * n * n * w - more // 2
+    srv.close()
+    srv = sgf.Server(hbm_budget=64 << 30, max_inflight=1, simulate_gbs=100.0, max_shape_bytes=whole - 1)
+    assert srv.submit(0, nest, prec, *arrays) == sgf.SGF_ENOMEM
+    srv.close()

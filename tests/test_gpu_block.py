@@ -170,3 +170,85 @@ def test_algorithmic_bytes_follow_the_reads(lib, n, levels, centre):
     nest = W.centred_nest(n, levels, centre=centre) if levels > 1 else W.Nest(n=n)
     plan = lib.Plan(nest, "fp32")
     assert plan.stats()["algorithmic_bytes"] == nest_pair_bytes([nest])["total"]
+
+
+# The root's one finer patch and one of that patch's two lie alike, centred in x: the products of the
+# root's pair sum mirror images over spectra that another target, of two sources, reads whole.
+SHARED_MIRROR = W.Forest(n=256, level=[0, 1, 2, 2], org=[(0, 0), (128, 0), (384, 0), (384, 256)])
+
+
+def test_mirror_images_over_spectra_read_whole_elsewhere(lib):
+    sigma = _sigma(SHARED_MIRROR, 13)
+    plan = lib.Plan(SHARED_MIRROR, "fp32")
+    gx, gy = run_gpu(plan, sigma)
+    samp = _sample(SHARED_MIRROR, 16, 7)
+    ox, oy = oracle.force_at(SHARED_MIRROR, sigma, *samp)
+    assert _worst(SHARED_MIRROR, (gx, gy), (ox, oy), samp) <= tol("fp32", 256)
+
+
+def _tol64(geom):
+    """FP64 bound of a nest: tol()'s 0.2 eps N^2 is that of lattice coordinates up to N; where levels m
+    apart meet they are those of the finer lattice, m times as large, and so are the corner
+    antiderivatives whose double differences leave the error (on both sides, oracle and tables)."""
+    return 2 ** (geom.levels - 1) * tol("fp64", geom.n)
+
+
+@pytest.mark.parametrize("name", ["256x3_odd", "300x3_embedded", "512x3_mirror_x", "2048x2"])
+def test_block_pairs_fp64_against_oracle(lib, name):
+    """B = 64 ... 256 and 1024, an instance of its own."""
+    geom = NESTS[name][0]
+    sigma = _sigma(geom, 3)
+    gx, gy = run_gpu(lib.Plan(geom, "fp64"), sigma)
+    samp = _sample(geom, 4 if geom.n >= 2048 else 16, 5)
+    ox, oy = oracle.force_at(geom, sigma, *samp)
+    assert _worst(geom, (gx, gy), (ox, oy), samp) <= _tol64(geom)
+
+
+@pytest.mark.parametrize("name,prec", [("256x3_odd", "fp64"), ("512x2_corner", "fp64"), ("300x3_embedded", "fp64"),
+                                       ("300x3_embedded", "fp32")])
+def test_block_potential_fp64_and_embedded(lib, name, prec):
+    geom = NESTS[name][0]
+    sigma = _sigma(geom, 4)
+    plan = lib.Plan(geom, prec, potential=True)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    phi = plan.solve_potential([torch.from_numpy(s).to(device="cuda", dtype=dt) for s in sigma])
+    torch.cuda.synchronize()
+    samp = _sample(geom, 16, 6)
+    ref = oracle.potential_at(geom, sigma, *samp)
+    worst = _worst(geom, ([p.double().cpu().numpy() for p in phi],), (ref,), samp)
+    assert worst <= (_tol64(geom) if prec == "fp64" else tol(prec, geom.n))
+
+
+@pytest.mark.parametrize("geom,prec,pot", [
+    (W.centred_nest(512, 2), "fp32", False), (W.centred_nest(256, 4, centre=(0.3, 0.0)), "fp32", False),  # side stream
+    (W.centred_nest(256, 2), "fp64", True), (W.two_patch_forest(256), "fp32", False),
+    (W.centred_nest(512, 3), "fp32", False), (W.centred_nest(1024, 2), "fp32", True)],  # one after the other
+    ids=["512x2", "256x4", "256x2_fp64_phi", "two_patches256", "512x3", "1024x2_phi"])
+def test_captured_block_solves_replay_bitwise(lib, geom, prec, pot):
+    """Captured into a graph before any eager solve, the side stream of small plans forked and joined
+    inside the capture; replayed on another stream than the capture's."""
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    plan = lib.Plan(geom, prec, potential=pot)
+    ts = [torch.from_numpy(s).to(device="cuda", dtype=dt) for s in _sigma(geom, 17)]
+    outs = [[torch.empty_like(t) for t in ts] for _ in range(1 if pot else 2)]
+    ptrs = [[t.data_ptr() for t in lst] for lst in [ts] + outs]
+    solve = plan.solve_potential_ptrs if pot else plan.solve_ptrs
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        solve(*ptrs)
+    torch.cuda.synchronize()
+    eager = [[torch.empty_like(t) for t in ts] for _ in outs]
+    for _ in range(2):
+        for lst in outs:
+            for t in lst:
+                t.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        solve(ptrs[0], *[[t.data_ptr() for t in lst] for lst in eager])
+        torch.cuda.synchronize()
+        for a, b in zip(outs, eager):
+            for x, y in zip(a, b):
+                assert torch.equal(x, y)

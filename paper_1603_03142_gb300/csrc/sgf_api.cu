@@ -614,8 +614,7 @@ int mac_units(const MacItem &it) { return it.m2 >> ((it.sym & kMirrorX ? 1 : 0) 
 // Work items of the products: targets whose terms read the same kernel spectra
 // share them, up to four right-hand sides an item, two where mirror images are summed
 // too (the accumulators of more do not fit in registers).  QG targets per warp
-// (mac_qg): fewer where the launch would leave SMs without warps (16 warps on each
-// of 152 SMs).  Mirror-symmetric items first, long ones before short ones.
+// (mac_qg): fewer where the launch would leave SMs without warps (16 on each).  Mirror-symmetric items first, long ones before short ones.
 void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &items, std::vector<MacTerm> &terms,
                std::vector<size_t> &xo, std::vector<size_t> &ao, MacLaunch *launch)
 {
@@ -670,7 +669,7 @@ void build_mac(const std::vector<BlkTarget> &tg, int vec, std::vector<MacItem> &
         long long warps = 0;
         for (const auto &it : items)
             warps += (long long)it.tiles * std::max(1, mac_units(it) / mac_qg(qg, it.rhs, it.sym));
-        if (warps >= 16 * 152)
+        if (warps >= 16 * kSMs)
             break;
     }
     for (auto &it : items) {

@@ -6,6 +6,7 @@
 namespace sgf {
 
 constexpr int kBlkThreads = 256;
+constexpr int kSMs = 152;  // of a GB300, for the rules that weigh a launch's CTAs or warps against them
 constexpr int kMaxStages = kMaxLevels - 1;
 enum : int { BLK_ROWS = 0, BLK_COLS = 1, BLK_ICOLS = 2, BLK_PASSES = 3, BLK_IROWS = 3 };
 

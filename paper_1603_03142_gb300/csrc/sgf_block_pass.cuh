@@ -105,8 +105,8 @@ cudaError_t blk_launch(int blocks, const SolveArgs<T> &a, const BlkArgs<T> &k, c
     if (blocks <= 0)
         return cudaSuccess;
     // forward rows: the three fields of a CTA's rows one after the other, or a CTA each where the
-    // launch would leave SMs without one (3 resident CTAs on each of 152 SMs)
-    const dim3 grid(blocks, PASS == BLK_ROWS && blocks < 3 * 152 ? 3 : 1);
+    // launch would leave SMs without one (3 resident CTAs on each)
+    const dim3 grid(blocks, PASS == BLK_ROWS && blocks < 3 * kSMs ? 3 : 1);
     k_blk<T, PASS, BATCH><<<grid, kBlkThreads, blk_smem<T>(PASS), st>>>(a, k, bt);
     return cudaGetLastError();
 }

@@ -1347,13 +1347,19 @@ size_t serial_inter_bytes(const sgf_plan *p)
     return std::max(align256(p->fwd_elems * Cb) + p->bwd_elems * Cb, p->blk_elems * Cb);
 }
 // Small solves, whose passes leave SMs idle: side by side they take (us, one after the
-// other / beside; centred nests) 256^2 2, 3 and 4 levels 80 / 60, 135 / 109, 245 / 233,
-// 512^2 2 levels 134 / 127.  Larger ones fill the SMs and lose what one part leaves in
+// other / beside; centred nests) 256^2 2, 3 and 4 levels 83 / 59, 131 / 105, 242 / 213,
+// 512^2 2 levels 137 / 113.  Larger ones fill the SMs and lose what one part leaves in
 // L2 for the next: 256^2 5 levels 591 / 631, 512^2 3 and 4 levels 298 / 342, 656 / 956,
-// 1024^2 3 levels 968 / 1193.
+// 1024^2 3 levels 968 / 1193.  So do forests of many 512^2 patches in FP32: 5 patches
+// 472 / 447, 6 621 / 653, 8 927 / 978 (potentials of 6 450 / 438, of 8 674 / 685), but at
+// 256^2 13 patches gain (715 / 674), and so do SGF_FP64 and SGF_BF16X, whose passes are
+// longer (512^2, 8 patches: 11770 / 11464, 1761 / 1675).
 bool blk_beside(const sgf_plan *p)
 {
-    return p->blk && (p->N <= 256 ? p->fo.depth <= 4 : p->N <= 512 && p->fo.depth == 2);
+    if (!p->blk || p->N > 512)
+        return false;
+    return p->N <= 256 ? p->fo.depth <= 4
+                       : p->fo.depth == 2 && (p->esize == 8 || p->tc || p->fo.K <= (p->pot ? 6 : 5));
 }
 size_t blk_offset(const sgf_plan *p)
 {

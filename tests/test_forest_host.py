@@ -91,3 +91,19 @@ def test_flags_on_forests():
     with pytest.raises(sgf.SgfError) as ei:
         sgf.estimate(W.Forest(n=4096, level=[0, 0], org=[(0, 0), (4096, 0)]), "bf16x")
     assert ei.value.status == sgf.SGF_EUNSUPPORTED
+
+
+@pytest.mark.parametrize("geom,prec,beside", [
+    (W.two_patch_forest(512), "fp32", True), (W.example3_forest(512), "fp32", False),
+    (W.example3_forest(512), "bf16x", True), (W.example3_forest(512), "fp64", True),
+    (W.example3_forest(256), "fp32", True), (W.two_patch_forest(1024), "fp32", False)])
+def test_workspace_where_block_passes_run_beside(geom, prec, beside):
+    """The block convolutions' fields take the place of the other intermediates where they run after
+    them, and follow them in small solves that run both at once; not in FP32 forests of many 512^2 patches."""
+    n, K, C = geom.n, geom.patches, 16 if prec == "fp64" else 8
+    own = K * (3 + 2) * (n + 1) * n * C  # forward slabs and column outputs of every patch
+    fields = K * 4 * (3 + 2) * (n // 2 + 1) * n * C  # every patch a source and a target of 4 units
+    covered = sum(bool(geom.covered_mask(p).any()) for p in range(K))
+    want = (own + fields if beside else max(own, fields)) + covered * n * n * C // 2
+    got = sgf.estimate(geom, prec)["workspace_bytes"]
+    assert want <= got <= want + (1 << 20)

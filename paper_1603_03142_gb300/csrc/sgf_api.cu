@@ -2638,11 +2638,12 @@ sgf_status autotune_impl(sgf_plan *p, int reps, cudaStream_t st, double ms[SGF_A
         dx[l] = base + (size_t)(p->L + l) * lal;
         dy[l] = base + (size_t)(2 * p->L + l) * lal;
     }
-    sgf_status s = solve_impl<T>(p, ds, dx, dy, st);  // fills the intermediates
+    void *const *fy = p->pot ? nullptr : dy;  // as the solves: an embedded potential plan stages no second result
+    sgf_status s = solve_impl<T>(p, ds, dx, fy, st);  // fills the intermediates
     if (s != SGF_OK)
         return s;
     SolveArgs<T> a;
-    fill_args<T>(p, ds, dx, dy, a, p->sched);
+    fill_args<T>(p, ds, dx, fy, a, p->sched);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if ((e = cudaEventCreate(&e0)) != cudaSuccess || (e = cudaEventCreate(&e1)) != cudaSuccess) {
         if (e0)
@@ -2750,7 +2751,7 @@ sgf_status autotune_impl(sgf_plan *p, int reps, cudaStream_t st, double ms[SGF_A
                 continue;
             p->sched = cand;
             SolveArgs<T> ac;
-            fill_args<T>(p, ds, dx, dy, ac, p->sched);
+            fill_args<T>(p, ds, dx, fy, ac, p->sched);
             s = timeit([&] { return launch_col<T>(p, ac, st); }, ms[c]);
         }
         p->sched = keep;
@@ -2763,7 +2764,7 @@ sgf_status autotune_impl(sgf_plan *p, int reps, cudaStream_t st, double ms[SGF_A
         for (int c = 0; c < 2 && s == SGF_OK; ++c) {
             p->sched.col_case3 = c;
             SolveArgs<T> ac;
-            fill_args<T>(p, ds, dx, dy, ac, p->sched);
+            fill_args<T>(p, ds, dx, fy, ac, p->sched);
             s = timeit([&] { return launch_col<T>(p, ac, st); }, ms[6 + c]);
         }
         p->sched = keep;

@@ -255,3 +255,18 @@ def test_zero_rim_potential_autotune(lib):
     ii, jj = rng.integers(0, n, 30), rng.integers(0, n, 30)
     ref = oracle.potential_at(nest, sigma, np.zeros_like(ii), ii, jj)
     assert np.abs(phi[jj, ii] - ref).max() <= tol("fp32", n) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n,levels,prec", [(24, 2, "fp64"), (300, 1, "fp32"), (300, 2, "fp64"), (600, 2, "fp32")])
+def test_embedded_potential_plans_tune(lib, n, levels, prec):
+    """The tuner solves once through the plan's embedding, which stages the densities and the one
+    result of a potential plan; a tuned plan's potential is the untuned one's to rounding."""
+    nest = W.centred_nest(n, levels) if levels > 1 else W.Nest(n=n)
+    sigma = _random_sigma(nest, 61)
+    plan = lib.Plan(nest, prec, potential=True)
+    before = run_phi(plan, sigma)
+    plan.autotune(reps=1)
+    after = run_phi(plan, sigma)
+    eps = np.finfo(np.float64 if prec == "fp64" else np.float32).eps
+    for a, b in zip(before, after):
+        assert np.abs(a - b).max() <= 64 * eps * np.abs(a).max()

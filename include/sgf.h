@@ -165,7 +165,12 @@ sgf_status sgf_plan_create(const sgf_nest_desc *desc, sgf_precision precision, s
  * intermediates, and for a plan over its spectra budget the generator's FP64
  * workspace), *spectra_bytes its kernel spectra (resident sets plus, over
  * budget, the window of the regenerated ones; shared between plans made by
- * sgf_plan_share).  The paper has no counterpart.  Errors: SGF_EINVAL. */
+ * sgf_plan_share).  Small nests and forests (up to four levels of n <= 256, two
+ * of n <= 512) solve their cross-level pairs beside their patches' own passes
+ * and hold the intermediates of both (256^2, three levels, SGF_FP32: 38 MiB in
+ * place of 31), a stream and two events, also where they only serve batches or
+ * sgf_solve_noalloc, which do not use them.  The paper has no counterpart.
+ * Errors: SGF_EINVAL. */
 sgf_status sgf_plan_footprint(const sgf_plan *plan, size_t *workspace_bytes, size_t *spectra_bytes);
 
 /* Plan options (bit flags) for sgf_plan_create_ex. */

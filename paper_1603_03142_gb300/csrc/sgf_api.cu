@@ -573,11 +573,16 @@ size_t blk_set_elems(const sgf_plan *p, const GenSet &g)
 }
 
 // Where the block transforms apply: nests (forests) of N >= 256 with blocks of at
-// least 16 cells (the smallest transform) at the plan's depth.  Below 256 the
-// whole-grid passes take fewer launches for transforms that are launch-bound
-// anyway, and so they do for FP32 potentials of a few patches on two levels at 256
-// (us per solve, whole-grid / block: 65.5 / 73.8; forces 76.8 / 79.1, but blocks save
-// a batch more; eight patches 556 / 327; three levels 258 / 147; FP64 forces 528 / 434).
+// least 16 cells (the smallest transform) at the plan's depth, but FP32 potentials of
+// a few patches on two levels at 256.  The line was drawn where the block passes'
+// launches outweighed what they save, before a small plan ran them beside its own
+// passes; as they run now, the whole-grid passes win at two levels below 256 and lose
+// from three on and at 256 (us per solve, whole grid / blocks: forces 64^2 2 levels
+// 39 / 45, 3 levels 86 / 73; 128^2 2 levels 43 / 49, 3 levels 111 / 74, two refined
+// patches 62 / 65, eight patches 221 / 119; 256^2 2 levels 77 / 60; potentials 128^2
+// 2 levels 39 / 49, 3 levels 96 / 70; 256^2 2 levels 66 / 56, two refined patches
+// 102 / 81; FP64 forces 128^2 2 levels 202 / 184; eight 128^2 nests in a batch, 2 levels
+// 150 / 108, 3 levels 618 / 212): it stands further out than it has to.
 // SGF_BF16X plans of three levels and more stay with the whole-grid passes: the
 // block transforms run in FP32, and from that depth on the split-BF16 rounding
 // they leave out moves the finest level's forces by up to 2.3e-5 (2-norm over 83
@@ -3167,7 +3172,9 @@ sgf_status sgf_solve_host(sgf_plan *p, const void *const *sigma, void *const *fx
     // CPU-GPU link, which saves the device-to-host copy; others are staged, and
     // so are all where the cross-level pairs add to the forces after that pass
     // (adding would read over the link what was just written; the crop of an
-    // embedded plan writes last, whatever came before).
+    // embedded plan writes last, whatever came before).  Page-locked buffers, us per
+    // call, whole-grid passes writing in place -> block convolutions copied out:
+    // 256^2 2 levels 112 -> 101, 1024^2 2 levels 656 -> 578, 3 levels 2179 -> 1224.
     const bool adds = p->blk && p->n_log == p->N;
     bool map_x[kMaxPatches], map_y[kMaxPatches];
     for (int l = 0; l < p->L; ++l) {

@@ -117,7 +117,9 @@ __device__ __forceinline__ void mac_body(const MacArgs<T> &m, const MacItem &it,
 // lane takes a frequency (kx, ky) and its mirror (kx, -ky), and every kernel value
 // serves its 2 or 4 mirror images: targets run over one half (quarter) of the units,
 // and half (a quarter) of the spectra are read.  Centred nests, the most common kind,
-// are symmetric in both axes: 1024^2 3 levels 627 -> 305 us for the products, 256^2 52 -> 38.
+// are symmetric in both axes: 1024^2 3 levels 627 -> 290 us for the products (5.2 of
+// 6.8 TB/s, held by load latency at 16 warps per SM: 128 registers, 8 bytes spilled),
+// 256^2, symmetric in y, 52 -> 38.
 // FP32: in FP64 the multiply-adds bound the products, not the spectra.
 template <int NC>
 __device__ constexpr bool mac_odd(bool y, int c, int f)

@@ -14,10 +14,10 @@
 // (N + 1) x 2N, read once per solve: the stage is bound by streaming them.
 //
 // Measured (FP32, GB300, us per solve; whole-grid passes -> this, with symmetric
-// products and the small solves' side stream): centred 1024^2 3 levels 2045 -> 978,
-// 2048^2 2 levels off centre 2214 -> 1752, 256^2 3 levels 280 -> 120, six 256^2
-// tiles and two refined patches 593 -> 304, 20 nests of 128 ... 1024 cells 3394 ->
-// 1650; the 2048^2 and the 20 nests' figures hold 81 us and 18 us of the column
+// products and the small solves' side stream): centred 1024^2 3 levels 2027 -> 952,
+// 2048^2 2 levels off centre 2208 -> 1751, 256^2 3 levels 278 -> 119, six 256^2
+// tiles and two refined patches 593 -> 305, 20 nests of 128 ... 1024 cells 3365 ->
+// 1628; the 2048^2 and the 20 nests' figures hold 81 us and 18 us of the column
 // pass's own gain (k_col_w).
 //
 // Passes of a solve, each one launch over every stage (one stage per m):

@@ -2590,6 +2590,12 @@ void tune_load_locked()
             w >= 0 && w <= 2)
             g_tune[key] = sgf_schedule{a, b, c, d, r, w};
     fclose(f);
+    // block convolutions without a line of their own (a file from before they had one) start from their size's
+    std::map<std::string, sgf_schedule> blk;
+    for (const auto &kv : g_tune)
+        if (kv.first.find("/ml1") != std::string::npos && kv.first.find("/blk") == std::string::npos)
+            blk.emplace(kv.first + "/blk", kv.second);
+    g_tune.insert(blk.begin(), blk.end());
 }
 
 void tune_store(const std::string &key, const sgf_schedule &s)

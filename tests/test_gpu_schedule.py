@@ -252,6 +252,29 @@ print(json.dumps({"first": first, "both": open(%r).read().split("\n")}))
     assert len(first) == 1 and len(both) == 2 and first[0] in both
 
 
+def test_block_plans_start_from_an_older_files_record(lib, tmp_path):
+    """A table file without a line for block convolutions: their plans start from the line of their
+    size and precision, as they did when there was one for both."""
+    import torch
+    dev = torch.cuda.get_device_name(0).replace(" ", "_")
+    table = tmp_path / "tune.txt"
+    table.write_text(f"{dev}/n256/p1/zr0/ml1 0 2 0 0 0 0\n{dev}/n512/p1/zr0/ml1 0 2 0 0 0 0\n"
+                     f"{dev}/n512/p1/zr0/ml1/blk 2 0 0 0 0 0\n")
+    code = r"""
+import sys, json
+sys.path.insert(0, %r)
+from paper_1603_03142_gb300 import sgf, workloads as W
+print(json.dumps([[p.schedule()["col_pass"], p.schedule()["row_inv0"]] for p in
+                  (sgf.Plan(W.centred_nest(256, 2), "fp32"), sgf.Plan(W.centred_nest(512, 2), "fp32"),
+                   sgf.Plan(W.centred_nest(128, 2), "fp32"))]))
+""" % str(ROOT)
+    env = dict(os.environ, SGF_AUTOTUNE_CACHE=str(table))
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0, out.stderr
+    import json
+    assert json.loads(out.stdout.strip().splitlines()[-1]) == [[0, 2], [2, 0], [0, 0]]
+
+
 @pytest.mark.parametrize("case", ["zero_rim_4096", "general_1024", "nest_512", "potential_1024"])
 def test_tma_gather_matches_lane_gather(lib, case):
     """row_inv0 = 3 (k_row_inv1t), 4 (k_row_inv1x) and 5 (k_row_inv2x) against
